@@ -659,6 +659,12 @@ int plan_create(cbs_plan_s** out, const cbs_plan_desc* desc, int seats) {
     const size_t row4 = (size_t)4 * a.rpb * a.nxp * sizeof(float2);
     a.nset_xf = (int)std::max<size_t>(2, std::min<size_t>(4, (kXBudget - fixed) / row4));
   }
+  // x axes that split into two radices run the warp-per-row passes (xrow.cu)
+  CKP(cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device));
+  const RowPlan rowp = plan_rows(d.nx, (long long)d.ny * d.nz, p->sms, 226 * 1024,
+                                 (size_t)twb[0] + 8 * 17 + 16 + 32 * 8);
+  if (rowp.A) CKP(xrow_set_smem_limit(d.nx, 227 * 1024));
+  a.xr = XRowShape{rowp.A, rowp.B, rowp.ldw, rowp.lde, rowp.rpb, rowp.sets, rowp.teams};
   // y and z tiles: TX columns x whole axis, brought in by boxes of B rows.  B is a divisor of
   // the axis in [16, 64] when one keeps every box's shared-memory offset (B TX 8 bytes) a
   // multiple of 128 bytes -- then no padded rows are held -- else 64 (rows past the axis
@@ -744,7 +750,7 @@ int plan_create(cbs_plan_s** out, const cbs_plan_desc* desc, int seats) {
     fail(CBS_ERR_CUDA, "cuTensorMapEncodeTiled failed for the workspace");
     return bail(CBS_ERR_CUDA);
   }
-  CKP(cudaMalloc(&p->partials, S * xpass_tiles(a) * sizeof(double)));   // >= seats x the x grid
+  CKP(cudaMalloc(&p->partials, S * std::max(xpass_tiles(a), a.xr.A ? xrow_tiles(a) : 0) * sizeof(double)));   // >= seats x the x grid
   CKP(cudaMalloc(&p->counter, S * sizeof(unsigned)));
   CKP(cudaMemset(p->counter, 0, S * sizeof(unsigned)));
   CKP(cudaMalloc(&p->hist, S * d.check_every * sizeof(double)));
@@ -781,6 +787,7 @@ int plan_create(cbs_plan_s** out, const cbs_plan_desc* desc, int seats) {
       std::vector<int4> st;
       std::vector<float2> tw, pq;
       axis_tables(n, p->radix_order[a2], st, tw, pq);
+      if (a2 == 0 && rowp.A) row_tables(n, rowp, tw, pq);
       std::copy(st.begin(), st.end(), st_all.begin() + a2 * 2 * kMaxAxisStages);
       twoff[a2] = (int)tw_all.size();
       tw.resize(round_up(n, 16), make_float2(0.f, 0.f));
@@ -811,11 +818,8 @@ int plan_create(cbs_plan_s** out, const cbs_plan_desc* desc, int seats) {
 
   // persistent grid sizes (occupancy of each tile kernel at its shared-memory size)
   {
-    int sms = 0;
-    CKP(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device));
-    p->sms = sms;
-    CKP(x_grid_size(a, sms));
-    CKP(yz_grid_sizes(a, sms));
+    CKP(x_grid_size(a, p->sms));
+    CKP(yz_grid_sizes(a, p->sms));
   }
 
   // every address the tile kernels bulk-copy from or to must be 16-byte aligned, every size

@@ -190,6 +190,137 @@ inline std::vector<int> order_radices_z(const std::vector<int>& radices, int n, 
   return best;
 }
 
+// --------------------------------------------------------------- x rows in two steps (xrow.cuh)
+// Instructions per value of a radix' in-register transform, roughly: what its split costs (the
+// odd primes' symmetric sums, one constant twiddle per value of a split).
+constexpr int radix_cost(int R) {
+  if (R <= 2) return R - 1;
+  if (R == 4) return 2;
+  for (int p : {4, 2, 3, 5, 7, 11, 13})
+    if (R % p == 0) return R == p ? p : radix_cost(p) + radix_cost(R / p) + 3;
+  return 1 << 20;
+}
+
+constexpr bool two_step_radix(int R) {
+  return (R >= 2 && R <= 16) || R == 18 || (R >= 20 && R <= 22) || (R >= 24 && R <= 28) || R == 30 || R == 32;
+}
+
+constexpr int row_pitch(int B) { return B + (6 - B % 4) % 4; }   // least pitch >= B that is 2 mod 4
+
+// Modelled work of a tile of rpb rows, whole rounds of 32 / B and 32 / A rows counted: step 1
+// (radix A) runs both transforms, the update and two twiddle products; step 2 (radix B) runs once
+// forward and once inverse, and a long one is dear: it holds B values between two warp barriers
+// and moves them as 16-byte pairs (640 on one plane of rows: 32 x 20 2.13 ms, 20 x 32 3.48 ms;
+// 275: 25 x 11 0.44 ms, 11 x 25 0.63 ms).
+constexpr int row_tile_cost(int A, int B, int rpb) {
+  const int per1 = 32 / B, per2 = 32 / A;
+  const int w1 = A * (2 * radix_cost(A) + 36), w2 = 2 * B * (radix_cost(B) + 2);
+  return (rpb + per1 - 1) / per1 * w1 + (rpb + per2 - 1) / per2 * (B > 16 ? w2 * 5 / 2 : w2);
+}
+
+// The larger radix A of the split n = A B an axis' kernels are built for (0: none): the least
+// work per row over tiles of 1, 2 and 4 rows that leave room for six of them (a row of an axis
+// too long for that is taken alone).
+constexpr int row_split(int n) {
+  int at = 0, least = 1 << 30;
+  for (int A = 32; A >= 2; --A) {
+    const int B = n / A;
+    if (A * B != n || !two_step_radix(A) || !two_step_radix(B)) continue;
+    for (int rpb = 1; rpb <= 4; rpb *= 2) {
+      if (rpb > 1 && 6 * rpb * 8 * (3 * A * row_pitch(B) + 4 * n) > 220 * 1024) continue;
+      const int c = row_tile_cost(A, B, rpb) * 4 / rpb;
+      if (c < least) {
+        least = c;
+        at = A;
+      }
+    }
+  }
+  return at;
+}
+
+struct RowPlan {
+  int A = 0, B = 0, ldw = 0, lde = 0, rpb = 0, sets = 0, teams = 0;
+};
+
+// Tile shape and pitches of an x axis of n with `rows` rows on `sms` processors.  fixed: bytes of
+// the tables; budget: shared memory of a block.  A = 0 when the axis has no split.
+inline RowPlan plan_rows(int n, long long rows, int sms, size_t budget, size_t fixed) {
+  RowPlan best;
+  const int A = row_split(n);
+  if (!A) return best;
+  const int B = n / A, P = row_pitch(B), even = (n + 1) / 2 * 2;
+  // pitches free of conflicts between the rows of a round: lanes over j (8-byte accesses), over
+  // k1 (16 bytes at pitch P) and over frequencies (8 bytes)
+  auto pitch = [&](int least, bool w) {
+    int at = least;
+    long long lowest = 1LL << 60;
+    for (int ld = least; ld < least + 16; ld += 2) {
+      long long addr[32], c = 0;
+      bool on[32];
+      auto fill = [&](int items, int step, int width) {
+        for (int l = 0; l < 32; ++l) {
+          on[l] = l / items < std::max(1, 32 / items);
+          addr[l] = 8LL * ((long long)(l / items) * ld + (long long)(l % items) * step);
+        }
+        c += warp_wavefronts(addr, on, width);
+      };
+      fill(B, 1, 8);
+      if (w) {
+        fill(A, P, 16);
+        fill(A, 1, 8);
+      }
+      if (c < lowest) {
+        lowest = c;
+        at = ld;
+      }
+    }
+    return at;
+  };
+  RowPlan p;
+  p.A = A;
+  p.B = B;
+  p.ldw = pitch(std::max(even, A * P), true);
+  p.lde = pitch(even, false);
+  // rows of a tile and teams: the least work of the busiest processor (its tiles times a tile's
+  // work and a tile's fixed part), with a set per team and one in flight unless a single row is
+  // too long for that.  Four teams where only they leave room for the better-filled rounds
+  // (384 = 24 x 16: two rows 0.665 ms, one row with five teams 0.771 ms), and one team less when
+  // the sets just suffice for single rows (640: 2.14 against 2.20 ms).
+  double least = 1e300;
+  for (int teams : {5, 4})
+    for (int rpb = 1; rpb <= 32; ++rpb) {
+      const size_t set = (size_t)rpb * (3 * p.ldw + 4 * p.lde) * 8;
+      const int sets = (int)std::min<size_t>(8, (budget - fixed) / set);
+      if (sets < 2 || (rpb > 1 && sets < teams + 1)) break;
+      p.rpb = rpb;
+      p.sets = sets;
+      p.teams = std::min(rpb == 1 && sets == teams + 1 ? teams - 1 : teams, sets - 1);
+      const long long tiles = (rows + rpb - 1) / rpb;
+      const double cost = (double)((tiles + sms - 1) / sms) * (row_tile_cost(A, B, rpb) + 50) * (teams == 4 ? 1.03 : 1.0);
+      if (cost < 0.99 * least) {
+        least = cost;
+        best = p;
+      }
+    }
+  return best;
+}
+
+// Twiddles w_n^{j k1} at k1 B + j and the wave numbers of the natural order, for plan_rows' axes.
+inline void row_tables(int n, const RowPlan& p, std::vector<float2>& tw, std::vector<float2>& pq) {
+  const double two_pi = 6.283185307179586476925287;
+  tw.clear();
+  for (int k = 0; k < p.A; ++k)
+    for (int j = 0; j < p.B; ++j) {
+      const double a = -two_pi * (double)((long long)j * k % n) / (double)n;
+      tw.push_back(make_float2((float)std::cos(a), (float)std::sin(a)));
+    }
+  pq.assign(n, make_float2(0.f, 0.f));
+  for (int k = 0; k < n; ++k) {
+    const float q = (float)(two_pi * (double)((2 * k < n) ? k : k - n) / (double)n);
+    pq[k] = make_float2(q, (2 * k == n) ? 0.f : q);
+  }
+}
+
 // Device tables of an axis for a given radix order (see fft_ip.cuh): the stage table
 // (2 int4 per stage), the twiddle table (complex64, w_n^{j k P_q} at tw_off_q + (k-1) m_q + j,
 // computed in FP64 and rounded), and the wave numbers (p, q) of each position (scaled by the

@@ -36,6 +36,13 @@ struct Member {
   int seat;               // slice of the plan's arrays: E, W at + seat * 3 Nw; V at + seat * Nw
 };
 
+// Shapes of the x passes of an axis nx = A B (xrow.cu); A = 0: the staged passes (xpass.cu).
+struct XRowShape {
+  int A, B;               // radices: x = j + B r, frequency k1 + A k2
+  int ldw, lde;           // row pitches of W, and of E and V, in a tile
+  int rpb, sets, teams;   // rows of a tile, tiles in shared memory, teams of three warps
+};
+
 // Everything one CBS iteration needs (kernel parameters, by value).
 struct IterArgs {
   int nx, ny, nz;
@@ -68,6 +75,7 @@ struct IterArgs {
   int slot;
   int* err;               // device error flag (a tensor-copy wait that timed out)
   // launch shapes
+  XRowShape xr;
   int rpb;                // rows per tile, x passes
   int nset_x, nset_xf;    // buffer sets of the x passes (inverse + forward; first forward)
   int tx_y, tx_z;         // x-columns per tile, y and z passes
@@ -107,6 +115,10 @@ cudaError_t launch_xpass_inv_fwd(const IterArgs& a, cudaStream_t s);  // IFFTx, 
 // Shared-memory bytes and threads of each pass for the plan's shapes.
 size_t xpass_smem(const IterArgs& a);
 int xpass_tiles(const IterArgs& a);
+size_t xrow_smem(const IterArgs& a);
+int xrow_tiles(const IterArgs& a);
+cudaError_t launch_xrow(const IterArgs& a, bool first, cudaStream_t s);   // both x passes of nx = A B
+cudaError_t xrow_set_smem_limit(int n, int bytes);
 cudaError_t yz_grid_sizes(IterArgs& a, int sms);   // sets grid_y, grid_z
 cudaError_t x_grid_size(IterArgs& a, int sms);     // sets grid_x, grid_xf
 

@@ -2,8 +2,8 @@
 //
 // The 3D FFTs of the CBS iteration (the "N log N" cost of Fig. 1(b) of arXiv 2506.15411)
 // are built from in-place DIF / DIT stages (fft_ip.cuh) whose butterflies are the DFTs below, applied to R values
-// held in registers.  Supported radices: 1 (identity), 2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12,
-// 13, 16.
+// held in registers.  Supported radices: 1 (identity) to 13 and 16, and for the kernels that
+// transform an axis in two steps also 14, 15, 18, 20, 21, 22, 24 to 28, 30 and 32.
 //   - odd primes: symmetric-pair form, X[k] and X[R-k] share the sums over the pairs
 //     x[m] +- x[R-m] with real cos/sin constants;
 //   - composites: one Cooley-Tukey split R = R1 * R2 (decimation in time) with the inner
@@ -222,7 +222,20 @@ template <bool INV> struct DFT<8, INV> : DFTSplit<2, 4, INV> {};
 template <bool INV> struct DFT<9, INV> : DFTSplit<3, 3, INV> {};
 template <bool INV> struct DFT<10, INV> : DFTSplit<2, 5, INV> {};
 template <bool INV> struct DFT<12, INV> : DFTSplit<3, 4, INV> {};
+template <bool INV> struct DFT<14, INV> : DFTSplit<2, 7, INV> {};
+template <bool INV> struct DFT<15, INV> : DFTSplit<3, 5, INV> {};
 template <bool INV> struct DFT<16, INV> : DFTSplit<4, 4, INV> {};
+template <bool INV> struct DFT<18, INV> : DFTSplit<2, 9, INV> {};
+template <bool INV> struct DFT<20, INV> : DFTSplit<4, 5, INV> {};
+template <bool INV> struct DFT<21, INV> : DFTSplit<3, 7, INV> {};
+template <bool INV> struct DFT<22, INV> : DFTSplit<2, 11, INV> {};
+template <bool INV> struct DFT<24, INV> : DFTSplit<3, 8, INV> {};
+template <bool INV> struct DFT<25, INV> : DFTSplit<5, 5, INV> {};
+template <bool INV> struct DFT<26, INV> : DFTSplit<2, 13, INV> {};
+template <bool INV> struct DFT<27, INV> : DFTSplit<3, 9, INV> {};
+template <bool INV> struct DFT<28, INV> : DFTSplit<4, 7, INV> {};
+template <bool INV> struct DFT<30, INV> : DFTSplit<5, 6, INV> {};
+template <bool INV> struct DFT<32, INV> : DFTSplit<4, 8, INV> {};
 
 // Calls f(std::integral_constant<int, R>) for the runtime radix r (uniform across the block).
 // Radices above MAXR are not compiled in (a plan whose axes need them uses a MAXR = 16
@@ -243,7 +256,20 @@ CBS_HD void radix_dispatch(int r, F&& f) {
     case 11: if constexpr (MAXR >= 11) f(std::integral_constant<int, 11>{}); break;
     case 12: if constexpr (MAXR >= 12) f(std::integral_constant<int, 12>{}); break;
     case 13: if constexpr (MAXR >= 13) f(std::integral_constant<int, 13>{}); break;
+    case 14: if constexpr (MAXR > 16) f(std::integral_constant<int, 14>{}); break;
+    case 15: if constexpr (MAXR > 16) f(std::integral_constant<int, 15>{}); break;
     case 16: if constexpr (MAXR >= 16) f(std::integral_constant<int, 16>{}); break;
+    case 18: if constexpr (MAXR >= 18) f(std::integral_constant<int, 18>{}); break;
+    case 20: if constexpr (MAXR >= 20) f(std::integral_constant<int, 20>{}); break;
+    case 21: if constexpr (MAXR >= 21) f(std::integral_constant<int, 21>{}); break;
+    case 22: if constexpr (MAXR >= 22) f(std::integral_constant<int, 22>{}); break;
+    case 24: if constexpr (MAXR >= 24) f(std::integral_constant<int, 24>{}); break;
+    case 25: if constexpr (MAXR >= 25) f(std::integral_constant<int, 25>{}); break;
+    case 26: if constexpr (MAXR >= 26) f(std::integral_constant<int, 26>{}); break;
+    case 27: if constexpr (MAXR >= 27) f(std::integral_constant<int, 27>{}); break;
+    case 28: if constexpr (MAXR >= 28) f(std::integral_constant<int, 28>{}); break;
+    case 30: if constexpr (MAXR >= 30) f(std::integral_constant<int, 30>{}); break;
+    case 32: if constexpr (MAXR >= 32) f(std::integral_constant<int, 32>{}); break;
     default: break;
   }
 }

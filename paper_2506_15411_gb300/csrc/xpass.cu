@@ -23,6 +23,7 @@
 #include "cbs_internal.h"
 #include "fft_ip.cuh"
 #include "tma.cuh"
+#include "xpass_common.cuh"
 
 namespace cbs {
 
@@ -41,46 +42,6 @@ __device__ __forceinline__ float2 source_at(const IterArgs& a, const SourceArgs&
     return cscale(__ldg(&s.user[c * a.N + idx]), s.user_scale);
   }
   return make_float2(0.f, 0.f);
-}
-
-// Block reduction of the per-thread residual in FP64, then a last-block-done pass that sums
-// the per-block partials of the request in seat `seat` (blocks b = 0 .. G-1 of its grid) in a
-// fixed order into its hist[slot] (deterministic).
-__device__ __forceinline__ void residual_finish(float acc, const IterArgs& a, int seat, int b, int G, double* wsum,
-                                                int* lastflag) {
-  double* const part = a.partials + (size_t)seat * a.grid_x;
-  unsigned* const counter = a.counter + seat;
-  double d = (double)acc;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) d += __shfl_down_sync(0xffffffffu, d, off);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int nw = (blockDim.x + 31) >> 5;
-  if (lane == 0) wsum[wid] = d;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double bs = 0.0;
-    for (int w = 0; w < nw; ++w) bs += wsum[w];
-    part[b] = bs;
-    __threadfence();
-    const unsigned prev = atomicAdd(counter, 1u);
-    *lastflag = (prev == (unsigned)G - 1);
-  }
-  __syncthreads();
-  if (!*lastflag) return;
-  __threadfence();
-  double s = 0.0;
-  for (int i = threadIdx.x; i < G; i += blockDim.x) s += __ldcg(&part[i]);
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-  __syncthreads();
-  if (lane == 0) wsum[wid] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double bs = 0.0;
-    for (int w = 0; w < nw; ++w) bs += wsum[w];
-    a.hist[(size_t)seat * a.hist_cap + a.slot] = bs;
-    *counter = 0u;
-  }
 }
 
 #ifndef CBS_X_THREADS
@@ -132,21 +93,6 @@ struct BlockSyncX {
 };
 
 __device__ __forceinline__ int x_tiles(const IterArgs& a) { return (a.ny * a.nz + a.rpb - 1) / a.rpb; }
-
-// (y, z) of memory row r of the y-blocked arrays: r = ((y / yblk) nz + z) yblk + y mod yblk
-struct RowDecode {
-  float inv_blk, inv_nz;
-  int blk, nz;
-  __device__ __forceinline__ void operator()(int r, int& y, int& z) const {
-    const int t = ip_div(r, inv_blk), yi = r - t * blk;
-    const int yb = ip_div(t, inv_nz);
-    z = t - yb * nz;
-    y = yb * blk + yi;
-  }
-};
-__device__ __forceinline__ RowDecode row_decode(const IterArgs& a) {
-  return RowDecode{1.0f / (float)a.yblk, 1.0f / (float)a.nz, a.yblk, a.nz};
-}
 
 // Row stages q0 .. q1-1 (forward) or q1-1 .. q0 (inverse) on ncomp x nr rows, a barrier after
 // each; `after_first` runs after the first barrier.
@@ -399,6 +345,10 @@ cudaError_t with_maxr_x(int maxr, F&& f) {
 // Persistent grids: as many blocks as fit at once (the inverse pass's, which is also the
 // number of residual partials), capped by the tile count.
 cudaError_t x_grid_size(IterArgs& a, int sms) {
+  if (a.xr.A) {
+    a.grid_x = a.grid_xf = std::max(1, std::min(xrow_tiles(a), sms));
+    return cudaSuccess;
+  }
   return with_maxr_x(a.maxr_x, [&](auto M) {
     constexpr int MR = decltype(M)::value;
     int occ_f = 0, occ_i = 0;
@@ -414,6 +364,7 @@ cudaError_t x_grid_size(IterArgs& a, int sms) {
 }
 
 cudaError_t launch_xpass_fwd(const IterArgs& a, cudaStream_t s) {
+  if (a.xr.A) return launch_xrow(a, true, s);
   return with_maxr_x(a.maxr_x, [&](auto M) {
     constexpr int MR = decltype(M)::value;
     k_xpass_fwd<MR><<<a.grid_xf * a.nmem, kThreads, xpass_fwd_smem(a), s>>>(a);
@@ -422,6 +373,7 @@ cudaError_t launch_xpass_fwd(const IterArgs& a, cudaStream_t s) {
 }
 
 cudaError_t launch_xpass_inv_fwd(const IterArgs& a, cudaStream_t s) {
+  if (a.xr.A) return launch_xrow(a, false, s);
   return with_maxr_x(a.maxr_x, [&](auto M) {
     constexpr int MR = decltype(M)::value;
     k_xpass_inv_fwd<MR><<<a.grid_x * a.nmem, kThreads, xpass_smem(a), s>>>(a);
