@@ -626,8 +626,6 @@ int plan_create(cbs_plan_s** out, const cbs_plan_desc* desc, int seats) {
   }
   CKP(cudaEventCreateWithFlags(&p->ev, cudaEventDisableTiming));
   CKP(cudaEventCreateWithFlags(&p->blk_ev, cudaEventDisableTiming));
-  CKP(xpass_set_smem_limit(227 * 1024));
-  CKP(yzpass_set_smem_limit(227 * 1024));
 
   IterArgs& a = p->base;
   a.nx = d.nx;
@@ -663,7 +661,7 @@ int plan_create(cbs_plan_s** out, const cbs_plan_desc* desc, int seats) {
   CKP(cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device));
   const RowPlan rowp = plan_rows(d.nx, (long long)d.ny * d.nz, p->sms, 226 * 1024,
                                  (size_t)twb[0] + 8 * 17 + 16 + 32 * 8);
-  if (rowp.A) CKP(xrow_set_smem_limit(d.nx, 227 * 1024));
+  CKP(rowp.A ? xrow_set_smem_limit(d.nx, 227 * 1024) : xpass_set_smem_limit(227 * 1024));
   a.xr = XRowShape{rowp.A, rowp.B, rowp.ldw, rowp.lde, rowp.rpb, rowp.sets, rowp.teams};
   // y and z tiles: TX columns x whole axis, brought in by boxes of B rows.  B is a divisor of
   // the axis in [16, 64] when one keeps every box's shared-memory offset (B TX 8 bytes) a
@@ -722,11 +720,30 @@ int plan_create(cbs_plan_s** out, const cbs_plan_desc* desc, int seats) {
     fail(CBS_ERR_ARG, "axis too long for the shared-memory tiles");
     return bail(CBS_ERR_ARG);
   }
+  // y and z axes that split into two radices run the two-step column passes (colpass.cuh)
+  ColPlan yp = col_plan(d.ny, 1);
+  const ColPlan zp = col_plan(d.nz, 3);
+  if (yp.A && !yblock_for(yp.tx)) yp = ColPlan{};
+  if (yp.A) {
+    a.tx_y = yp.tx;
+    const int blk = yblock_for(yp.tx);
+    const int sets = (kColSmem - col_fixed_smem(d.ny, 1)) / (d.ny * yp.tx * (int)sizeof(float2));
+    a.yc = ColShape{std::min(8, sets), blk, d.ny / blk, yp.threads(), yp.tx};
+    CKP(col_set_smem_limit(d.ny, false, 227 * 1024));
+  }
+  if (zp.A) {
+    a.tx_z = zp.tx;
+    const int box = z_box_rows(d.nz, zp.tx), nb = (d.nz + 255) / 256;
+    const int sets = (kColSmem - col_fixed_smem(d.nz, 3)) / (3 * nb * box * zp.tx * (int)sizeof(float2));
+    a.zc = ColShape{std::min(8, sets), box, nb, zp.threads(), zp.tx};
+    CKP(col_set_smem_limit(d.nz, true, 227 * 1024));
+  }
+  if (!yp.A || !zp.A) CKP(yzpass_set_smem_limit(227 * 1024));
   a.yblk = yblock_for(a.tx_y);
   a.nyb = d.ny / a.yblk;
   a.yb = a.yblk;
   a.nyr = d.ny;
-  a.zb = box_rows(d.nz, a.tx_z);
+  a.zb = a.zc.sets ? a.zc.box : box_rows(d.nz, a.tx_z);
   a.nzr = round_up(d.nz, a.zb);
   a.maxr_x = max_radix(rad[0]);
   a.maxr_z = max_radix(rad[2]);
@@ -782,12 +799,16 @@ int plan_create(cbs_plan_s** out, const cbs_plan_desc* desc, int seats) {
     int twoff[3], pqoff[3];
     for (int a2 = 0; a2 < 3; ++a2) {
       const int n = dims[a2];
-      p->radix_order[a2] = a2 == 2 ? order_radices_z(rad[a2], n, a.tx_z, kZThreadsPlan / a.zgroups)
-                                   : order_radices(rad[a2], n, lay[a2], ncol[a2]);
+      const bool two_step = a2 == 0 ? rowp.A > 0 : (a2 == 1 ? yp.A > 0 : zp.A > 0);
+      p->radix_order[a2] = two_step  ? rad[a2]   // (only the staged passes use it)
+                           : a2 == 2 ? order_radices_z(rad[a2], n, a.tx_z, kZThreadsPlan / a.zgroups)
+                                     : order_radices(rad[a2], n, lay[a2], ncol[a2]);
       std::vector<int4> st;
       std::vector<float2> tw, pq;
       axis_tables(n, p->radix_order[a2], st, tw, pq);
       if (a2 == 0 && rowp.A) row_tables(n, rowp, tw, pq);
+      if (a2 == 1 && yp.A) col_tables(n, yp, true, tw, pq);
+      if (a2 == 2 && zp.A) col_tables(n, zp, false, tw, pq);
       std::copy(st.begin(), st.end(), st_all.begin() + a2 * 2 * kMaxAxisStages);
       twoff[a2] = (int)tw_all.size();
       tw.resize(round_up(n, 16), make_float2(0.f, 0.f));

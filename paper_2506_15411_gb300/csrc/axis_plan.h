@@ -238,6 +238,90 @@ constexpr int row_split(int n) {
   return at;
 }
 
+// ------------------------------------------------------- columns in two steps (colpass.cuh)
+struct ColPlan {
+  int A = 0, tx = 0, gt = 0, groups = 0;   // n = A B, columns of a tile, threads of a group, groups
+  constexpr int threads() const { return groups * gt + 32; }
+};
+
+// Rows of a tensor-copy box of a z tile: the axis in as few boxes as fit (256 rows), each a
+// multiple of 128 bytes in shared memory.
+constexpr int z_box_rows(int n, int tx) {
+  const int nb = (n + 255) / 256, rows = (n + nb - 1) / nb;
+  return tx == 8 ? (rows + 1) / 2 * 2 : rows;
+}
+// Shared memory of a block but its tiles: twiddles, wave numbers (z), mbarriers and flags.
+constexpr int col_fixed_smem(int n, int ncomp) { return (n + 1) / 2 * 16 * (ncomp == 3 ? 2 : 1) + 8 * 17 + 48; }
+constexpr int kColSmem = 226 * 1024;
+
+// Shape of the y (ncomp = 1) or z (3) kernels of an axis of n; A = 0: none.  Radices up to 32 (z:
+// 36 and 12, as step 2 holds three components).  Least modelled time per value: the instructions
+// of a group's rounds over a tile's items, at the third of an instruction per cycle that a warp
+// issues alone and shared by the groups, plus those of all warps at three per cycle.  Threads
+// are kept few enough for the values a thread holds (z of 336 = 28 x 12, 27 million voxels: two
+// groups of 288 threads spill at 96 registers, 0.34 ms; of 224, 0.29 ms).  y passes wait for memory,
+// so two sets beyond the groups' and tiles of 16 columns count for more there (384: 0.29 against
+// 0.31 ms), and so does A < B, whose first step leaves step 2 the shorter rounds (640, forward:
+// 20 x 32 1.10 ms, 32 x 20 1.37 ms).
+constexpr ColPlan col_plan(int n, int ncomp) {
+  ColPlan best;
+  double least = 1e300;
+  for (int tx = 16; tx >= 8; tx /= 2) {
+    if (ncomp == 1 && tx == 8 && n % 2) continue;   // (y boxes must keep 128-byte offsets)
+    const int rows = ncomp == 3 ? z_box_rows(n, tx) * ((n + 255) / 256) : n;
+    int sets = (kColSmem - col_fixed_smem(n, ncomp)) / (ncomp * rows * tx * 8);
+    if (sets > 8) sets = 8;
+    if (sets < 3) continue;
+    for (int A = 2; A <= 36; ++A) {
+      const int B = n / A;
+      if (A * B != n || !two_step_radix(B)) continue;
+      if (ncomp == 3 ? (B > 12 || !(two_step_radix(A) || A == 35 || A == 36)) : !two_step_radix(A)) continue;
+      const int regs = (A > ncomp * B ? A : ncomp * B) * 2;
+      const int most = regs > 64 ? 512 : (regs > 50 ? 608 : 736);   // threads: at least 128, 96 or 80 registers
+      const double w1 = A * (radix_cost(A) + 8.0) * (ncomp == 3 ? 2 : 1);
+      const double w2 = ncomp == 1 ? B * (radix_cost(B) + 3.0) : 6.0 * B * (radix_cost(B) + 2.0) + 34.0 * B;
+      const int i1 = ncomp * tx * B, i2 = tx * A;
+      for (int gt = 64; gt <= 320; gt += 32) {
+        int groups = (most - 32) / gt;
+        if (groups > sets - 1) groups = sets - 1;
+        if (groups > 6) groups = 6;
+        if (groups < 1) continue;
+        const double alone = ((i1 + gt - 1) / gt * w1 + (i2 + gt - 1) / gt * w2 + 150.0) * 3.0 / groups;
+        const double issue = ((i1 + 31) / 32 * w1 + (i2 + 31) / 32 * w2) / 3.0;
+        const double cost = (alone + issue) / (n * tx) * 
+                            (ncomp == 1 ? (sets - groups >= 2 ? 1.0 : 1.2) * (tx == 8 ? 1.2 : 1.0) * (A > B ? 1.1 : 1.0) : 1.0);
+        if (cost < 0.995 * least) {
+          least = cost;
+          best.A = A;
+          best.tx = tx;
+          best.gt = gt;
+          best.groups = groups;
+        }
+      }
+    }
+  }
+  return best;
+}
+
+// Tables of a column axis: twiddles w_n^{j k1} at k1 B + j; wave numbers by row (y: frequency
+// k1 + A k2 sits in row k1 B + (k2 ^ s), s = k1 & 1 for 8 columns and even B) or by frequency (z).
+inline void col_tables(int n, const ColPlan& p, bool by_row, std::vector<float2>& tw, std::vector<float2>& pq) {
+  const double two_pi = 6.283185307179586476925287;
+  const int A = p.A, B = n / A;
+  tw.clear();
+  for (int k = 0; k < A; ++k)
+    for (int j = 0; j < B; ++j) {
+      const double a = -two_pi * (double)((long long)j * k % n) / (double)n;
+      tw.push_back(make_float2((float)std::cos(a), (float)std::sin(a)));
+    }
+  pq.assign(n, make_float2(0.f, 0.f));
+  for (int k = 0; k < n; ++k) {
+    const int k1 = k % A, k2 = k / A, s = (p.tx == 8 && B % 2 == 0) ? k1 & 1 : 0;
+    const float q = (float)(two_pi * (double)((2 * k < n) ? k : k - n) / (double)n);
+    pq[by_row ? k1 * B + (k2 ^ s) : k] = make_float2(q, (2 * k == n) ? 0.f : q);
+  }
+}
+
 struct RowPlan {
   int A = 0, B = 0, ldw = 0, lde = 0, rpb = 0, sets = 0, teams = 0;
 };

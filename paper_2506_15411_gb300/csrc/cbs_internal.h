@@ -43,6 +43,13 @@ struct XRowShape {
   int rpb, sets, teams;   // rows of a tile, tiles in shared memory, teams of three warps
 };
 
+// Shapes of the column passes of an axis n = A B (colpass.cuh); sets = 0: the staged passes.
+struct ColShape {
+  int sets;               // tiles in shared memory
+  int box, nbox;          // rows of a tensor-copy box, boxes of a component
+  int threads, tx;
+};
+
 // Everything one CBS iteration needs (kernel parameters, by value).
 struct IterArgs {
   int nx, ny, nz;
@@ -76,6 +83,7 @@ struct IterArgs {
   int* err;               // device error flag (a tensor-copy wait that timed out)
   // launch shapes
   XRowShape xr;
+  ColShape yc, zc;
   int rpb;                // rows per tile, x passes
   int nset_x, nset_xf;    // buffer sets of the x passes (inverse + forward; first forward)
   int tx_y, tx_z;         // x-columns per tile, y and z passes
@@ -119,6 +127,8 @@ size_t xrow_smem(const IterArgs& a);
 int xrow_tiles(const IterArgs& a);
 cudaError_t launch_xrow(const IterArgs& a, bool first, cudaStream_t s);   // both x passes of nx = A B
 cudaError_t xrow_set_smem_limit(int n, int bytes);
+cudaError_t launch_col(const CUtensorMap& tm, const IterArgs& a, int kind, cudaStream_t s);   // y, inverse y, z
+cudaError_t col_set_smem_limit(int n, bool z, int bytes);
 cudaError_t yz_grid_sizes(IterArgs& a, int sms);   // sets grid_y, grid_z
 cudaError_t x_grid_size(IterArgs& a, int sms);     // sets grid_x, grid_xf
 

@@ -3,7 +3,7 @@
 // The 3D FFTs of the CBS iteration (the "N log N" cost of Fig. 1(b) of arXiv 2506.15411)
 // are built from in-place DIF / DIT stages (fft_ip.cuh) whose butterflies are the DFTs below, applied to R values
 // held in registers.  Supported radices: 1 (identity) to 13 and 16, and for the kernels that
-// transform an axis in two steps also 14, 15, 18, 20, 21, 22, 24 to 28, 30 and 32.
+// transform an axis in two steps also 14, 15, 18, 20, 21, 22, 24 to 28, 30, 32, 35 and 36.
 //   - odd primes: symmetric-pair form, X[k] and X[R-k] share the sums over the pairs
 //     x[m] +- x[R-m] with real cos/sin constants;
 //   - composites: one Cooley-Tukey split R = R1 * R2 (decimation in time) with the inner
@@ -236,6 +236,8 @@ template <bool INV> struct DFT<27, INV> : DFTSplit<3, 9, INV> {};
 template <bool INV> struct DFT<28, INV> : DFTSplit<4, 7, INV> {};
 template <bool INV> struct DFT<30, INV> : DFTSplit<5, 6, INV> {};
 template <bool INV> struct DFT<32, INV> : DFTSplit<4, 8, INV> {};
+template <bool INV> struct DFT<35, INV> : DFTSplit<5, 7, INV> {};
+template <bool INV> struct DFT<36, INV> : DFTSplit<4, 9, INV> {};
 
 // Calls f(std::integral_constant<int, R>) for the runtime radix r (uniform across the block).
 // Radices above MAXR are not compiled in (a plan whose axes need them uses a MAXR = 16
@@ -270,6 +272,8 @@ CBS_HD void radix_dispatch(int r, F&& f) {
     case 28: if constexpr (MAXR >= 28) f(std::integral_constant<int, 28>{}); break;
     case 30: if constexpr (MAXR >= 30) f(std::integral_constant<int, 30>{}); break;
     case 32: if constexpr (MAXR >= 32) f(std::integral_constant<int, 32>{}); break;
+    case 35: if constexpr (MAXR >= 35) f(std::integral_constant<int, 35>{}); break;
+    case 36: if constexpr (MAXR >= 36) f(std::integral_constant<int, 36>{}); break;
     default: break;
   }
 }

@@ -34,9 +34,18 @@ int zpass_tiles(const IterArgs& a) { return (a.nx + a.tx_z - 1) / a.tx_z * a.ny;
 // Persistent grids: as many blocks as fit on the device at once (capped by the tile count).
 cudaError_t yz_grid_sizes(IterArgs& a, int sms) {
   int occ = 0;
-  cudaError_t e = with_tx(a.tx_y, [&](auto T) { return y_occupancy<decltype(T)::value>(a, &occ); });
+  cudaError_t e = cudaSuccess;
+  if (a.yc.sets) {   // one block per SM
+    a.grid_y = std::max(1, std::min(ypass_tiles(a), sms));
+  } else {
+  e = with_tx(a.tx_y, [&](auto T) { return y_occupancy<decltype(T)::value>(a, &occ); });
   if (e != cudaSuccess) return e;
   a.grid_y = std::max(1, std::min(ypass_tiles(a), sms * std::max(1, occ)));
+  }
+  if (a.zc.sets) {
+    a.grid_z = std::max(1, std::min(zpass_tiles(a), sms));
+    return cudaSuccess;
+  }
   e = with_tx(a.tx_z, [&](auto T) { return z_occupancy<decltype(T)::value>(a, &occ); });
   if (e != cudaSuccess) return e;
   a.grid_z = std::max(1, std::min(zpass_tiles(a), sms * std::max(1, occ)));
@@ -44,10 +53,12 @@ cudaError_t yz_grid_sizes(IterArgs& a, int sms) {
 }
 
 cudaError_t launch_ypass(const CUtensorMap& tm, const IterArgs& a, bool inverse, cudaStream_t s) {
+  if (a.yc.sets) return launch_col(tm, a, inverse ? 1 : 0, s);
   return with_tx(a.tx_y, [&](auto T) { return y_launch<decltype(T)::value>(tm, a, inverse, s); });
 }
 
 cudaError_t launch_zpass_green(const CUtensorMap& tm, const IterArgs& a, cudaStream_t s) {
+  if (a.zc.sets) return launch_col(tm, a, 2, s);
   return with_tx(a.tx_z, [&](auto T) { return z_launch<decltype(T)::value>(tm, a, s); });
 }
 

@@ -1,4 +1,4 @@
-"""The two-step x passes (csrc/xrow.cuh) on every axis length they take, against
+"""The two-step passes (csrc/xrow.cuh, csrc/colpass.cuh) on every axis length they take, against
 the FP64 oracle: one axis runs over all lengths that split into two radices while the others are
 short and odd, so that tiles, lanes and boxes have remainders in every shape.  Tolerance: three
 complex64 iterations carry about 1e-6 each (six short transforms of length <= 1024 and a dozen
@@ -51,6 +51,20 @@ def _check(nx, ny, nz):
 def test_every_x_length(lo, hi):
     for n in _lengths(lo, hi):
         _check(n, 7, 3 if n % 2 else 5)
+
+
+@pytest.mark.parametrize("lo,hi", [(4, 128), (129, 400), (401, 1024)])
+def test_every_y_length(lo, hi):
+    for n in _lengths(lo, hi):
+        if n % 2 and n > 853:
+            continue    # refused: two tiles of 16 columns, the only width for odd y, do not fit
+        _check(18 if n % 2 else 9, n, 3)
+
+
+@pytest.mark.parametrize("lo,hi", [(4, 128), (129, 432)])
+def test_every_z_length(lo, hi):
+    for n in _lengths(lo, hi):
+        _check(9 if n % 2 else 18, 3, n)
 
 
 @pytest.mark.parametrize("grid", [(40, 132, 64), (45, 56, 130), (96, 270, 63)])
