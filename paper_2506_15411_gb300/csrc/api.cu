@@ -406,7 +406,7 @@ void series_begin(cbs_plan_s* p, float2* E, const SourceArgs& src, int warm, Ser
   if (warm == 2) {
     IterArgs a1 = R.a;
     a1.slot = 0;
-    int rc = launch_xpass_fwd(a1, p->stream) == cudaSuccess ? CBS_OK : fail(CBS_ERR_CUDA, "x pass launch failed");
+    int rc = launch_xpass_fwd(a1, true, p->stream) == cudaSuccess ? CBS_OK : fail(CBS_ERR_CUDA, "x pass launch failed");
     if (!rc) rc = launch_iteration(p, a1, p->stream, nullptr);
     if (!rc) {
       e = cudaMemcpyAsync(p->hist_host, p->hist, sizeof(double), cudaMemcpyDeviceToHost, p->stream);
@@ -428,7 +428,7 @@ void series_begin(cbs_plan_s* p, float2* E, const SourceArgs& src, int warm, Ser
   }
   if (warm && e == cudaSuccess)
     e = field_copy(p, 0, E, false, p->stream);
-  if (e == cudaSuccess) e = launch_xpass_fwd(R.a, p->stream);   // W of the first iteration
+  if (e == cudaSuccess) e = launch_xpass_fwd(R.a, warm == 0, p->stream);   // W of the first iteration
   if (e != cudaSuccess) {
     R.rc = fail(CBS_ERR_CUDA, "field copy-in: %s", cudaGetErrorString(e));
     R.finished = true;
@@ -535,34 +535,18 @@ namespace cbs {
 // |k^2 - k0^2| over the grid (absorbing layers included), V = k^2 - k0^2 - i epsilon in the
 // seat's slice.  The scaled k0^2 and epsilon land in seat_k0sq / seat_eps.
 int seat_permittivity(cbs_plan_s* p, int seat, const float* eps, cudaStream_t s) {
-  const int B = p->red_blocks;
-  CK(launch_eps_minmax(eps, p->N, p->pmin, p->pmax, p->pbad, B, s));
-  std::vector<float> mn(B), mx(B);
-  std::vector<int> bad(B);
-  CK(cudaMemcpyAsync(mn.data(), p->pmin, B * sizeof(float), cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(mx.data(), p->pmax, B * sizeof(float), cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(bad.data(), p->pbad, B * sizeof(int), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
-  double lo = 1e300, hi = -1e300;
-  for (int b = 0; b < B; ++b) {
-    if (bad[b]) return fail(CBS_ERR_ARG, "permittivity contains a non-finite value");
-    lo = std::min(lo, (double)mn[b]);
-    hi = std::max(hi, (double)mx[b]);
-  }
   const double kv2 = (p->kvac * p->pitch) * (p->kvac * p->pitch);
-  const double k0sq = 0.5 * kv2 * (lo + hi);
-  CK(launch_k2_maxdev(eps, p->d.nx, p->d.ny, p->d.nz, p->sx, p->sy, p->sz, p->layers.corner_max, kv2, k0sq,
-                      p->pdev, B, s));
-  std::vector<double> dv(B);
-  CK(cudaMemcpyAsync(dv.data(), p->pdev, B * sizeof(double), cudaMemcpyDeviceToHost, s));
+  const int xlo = p->d.pad_lo[0], xhi = p->d.nx - p->d.pad_hi[0];
+  CK(launch_splitting(eps, p->d.nx, p->d.ny, p->d.nz, xlo, xhi, p->sx, p->sy, p->sz, p->layers.corner_max, kv2, p->pmin,
+                      p->pmax, p->pbad, p->pdev, p->red_blocks, p->split, s));
+  CK(launch_build_v(eps, p->d.nx, p->d.ny, p->d.nz, p->base.nxp, p->base.yblk, xlo, xhi, p->sx, p->sy, p->sz,
+                    p->layers.corner_max, kv2, p->split, p->V + (size_t)seat * p->base.Nw, s));
+  CK(cudaMemcpyAsync(p->split_host, p->split, sizeof(Splitting), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
-  double epsilon = 0.0;
-  for (int b = 0; b < B; ++b) epsilon = std::max(epsilon, dv[b]);
+  const double k0sq = p->split_host->k0sq, epsilon = p->split_host->eps;
+  if (p->split_host->bad) return fail(CBS_ERR_ARG, "permittivity contains a non-finite value");
   if (!(epsilon > 0.0) || !std::isfinite(epsilon))
     return fail(CBS_ERR_ARG, "epsilon = %g: a lossless homogeneous grid has no convergent splitting", epsilon);
-  CK(launch_build_v(eps, p->d.nx, p->d.ny, p->d.nz, p->base.nxp, p->base.yblk, p->sx, p->sy, p->sz,
-                    p->layers.corner_max, kv2, k0sq, epsilon, p->V + (size_t)seat * p->base.Nw, s));
-  CK(cudaStreamSynchronize(s));
   p->seat_k0sq[seat] = k0sq;
   p->seat_eps[seat] = epsilon;
   return CBS_OK;
@@ -786,6 +770,9 @@ int plan_create(cbs_plan_s** out, const cbs_plan_desc* desc, int seats) {
   CKP(cudaMalloc(&p->pmax, p->red_blocks * sizeof(float)));
   CKP(cudaMalloc(&p->pbad, p->red_blocks * sizeof(int)));
   CKP(cudaMalloc(&p->pdev, p->red_blocks * sizeof(double)));
+  CKP(cudaMalloc(&p->split, sizeof(Splitting)));
+  CKP(cudaMemset(p->split, 0, sizeof(Splitting)));
+  CKP(cudaMallocHost(&p->split_host, sizeof(Splitting)));
 
   // per-axis FFT tables (axis_plan.h): radix order for the axis' shared-memory layout, stage
   // table, per-stage twiddles (FP64, rounded; padded to n entries so that a fixed n * 8 bytes
@@ -900,11 +887,12 @@ void cbs_destroy(cbs_plan_t p) {
   drop_graphs(p);
   void* devs[] = {p->V, p->W, p->Ei, p->tw, p->pq, p->stages, p->partials, p->counter, p->hist, p->mem_dev,
                   p->adj_amp, p->dobj,
-                  p->sx, p->sy, p->sz, p->pmin, p->pmax, p->pbad, p->pdev, p->eps_dev,
+                  p->sx, p->sy, p->sz, p->pmin, p->pmax, p->pbad, p->pdev, p->split, p->eps_dev,
                   p->Ef, p->Ea, p->grad_dev, p->err_dev};
   for (void* q : devs)
     if (q) cudaFree(q);
   if (p->hist_host) cudaFreeHost(p->hist_host);
+  if (p->split_host) cudaFreeHost(p->split_host);
   if (p->mem_host) cudaFreeHost(p->mem_host);
   if (p->err_host) cudaFreeHost(p->err_host);
   if (p->ev) cudaEventDestroy(p->ev);

@@ -115,7 +115,7 @@ CBS_HD size_t wrow(int y, int z, int nz, int yblk) {
 }
 
 // Launchers (one per pass of an iteration); each returns the launch error.
-cudaError_t launch_xpass_fwd(const IterArgs& a, cudaStream_t s);   // W = FFTx(V E + S)
+cudaError_t launch_xpass_fwd(const IterArgs& a, bool zero, cudaStream_t s);   // W = FFTx(V E + S); zero: E is 0
 cudaError_t launch_ypass(const CUtensorMap& tm, const IterArgs& a, bool inverse, cudaStream_t s);
 cudaError_t launch_zpass_green(const CUtensorMap& tm, const IterArgs& a, cudaStream_t s);  // FFTz, G, IFFTz
 cudaError_t launch_xpass_inv_fwd(const IterArgs& a, cudaStream_t s);  // IFFTx, update, residual, next FFTx
@@ -125,7 +125,7 @@ size_t xpass_smem(const IterArgs& a);
 int xpass_tiles(const IterArgs& a);
 size_t xrow_smem(const IterArgs& a);
 int xrow_tiles(const IterArgs& a);
-cudaError_t launch_xrow(const IterArgs& a, bool first, cudaStream_t s);   // both x passes of nx = A B
+cudaError_t launch_xrow(const IterArgs& a, int mode, cudaStream_t s);   // the x passes of nx = A B
 cudaError_t xrow_set_smem_limit(int n, int bytes);
 cudaError_t launch_col(const CUtensorMap& tm, const IterArgs& a, int kind, cudaStream_t s);   // y, inverse y, z
 cudaError_t col_set_smem_limit(int n, bool z, int bytes);
@@ -133,14 +133,19 @@ cudaError_t yz_grid_sizes(IterArgs& a, int sms);   // sets grid_y, grid_z
 cudaError_t x_grid_size(IterArgs& a, int sms);     // sets grid_x, grid_xf
 
 // Set-up and gradient kernels (misc.cu).
-cudaError_t launch_eps_minmax(const float* eps, size_t N, float* part_min, float* part_max,
-                              int* part_bad, int blocks, cudaStream_t s);
-cudaError_t launch_k2_maxdev(const float* eps, int nx, int ny, int nz, const double* sx,
-                             const double* sy, const double* sz, int corner_max, double kv2, double k0sq,
-                             double* part, int blocks, cudaStream_t s);
-cudaError_t launch_build_v(const float* eps, int nx, int ny, int nz, int nxp, int yblk, const double* sx,
-                           const double* sy, const double* sz, int corner_max, double kv2, double k0sq,
-                           double eps_shift, float2* V, cudaStream_t s);
+// The splitting of a permittivity as the set-up kernels leave it on the device.
+struct Splitting {
+  double k0sq, eps;       // scaled k0^2 and epsilon
+  int bad;                // a non-finite permittivity
+  unsigned count;         // last-block counter (left at 0)
+};
+// xlo .. xhi - 1: the voxels along x outside the absorbing layers
+cudaError_t launch_splitting(const float* eps, int nx, int ny, int nz, int xlo, int xhi, const double* sx, const double* sy,
+                             const double* sz, int corner_max, double kv2, float* pmin, float* pmax, int* pbad,
+                             double* part, int blocks, Splitting* sp, cudaStream_t s);
+cudaError_t launch_build_v(const float* eps, int nx, int ny, int nz, int nxp, int yblk, int xlo, int xhi, const double* sx,
+                           const double* sy, const double* sz, int corner_max, double kv2, const Splitting* sp,
+                           float2* V, cudaStream_t s);
 // A field between the caller's dense layout [3][nz][ny][nx] and the plan's y-blocked one
 // (to_dense: plan -> dense); the row padding of the plan's copy is not written.
 cudaError_t launch_field_layout(const float2* src, float2* dst, bool to_dense, int nx, int ny, int nz, int nxp,

@@ -96,6 +96,8 @@ struct cbs_plan_s {
   int* pbad = nullptr;
   double* pdev = nullptr;
   int red_blocks = 0;
+  cbs::Splitting* split = nullptr;       // the splitting on the device, and its pinned copy
+  cbs::Splitting* split_host = nullptr;
   // host staging (pinned)
   double* hist_host = nullptr;
   // host-buffer design step

@@ -264,7 +264,7 @@ int seat_begin(Batch* b, Seat& s, float2* E, const SourceArgs& src, Phase phase)
   IterArgs a = p->base;
   a.nmem = 1;
   a.mem = p->mem_dev + 1 + s.idx;
-  CK(launch_xpass_fwd(a, b->stream));
+  CK(launch_xpass_fwd(a, true, b->stream));
   s.phase = phase;
   return CBS_OK;
 }

@@ -363,8 +363,8 @@ cudaError_t x_grid_size(IterArgs& a, int sms) {
   });
 }
 
-cudaError_t launch_xpass_fwd(const IterArgs& a, cudaStream_t s) {
-  if (a.xr.A) return launch_xrow(a, true, s);
+cudaError_t launch_xpass_fwd(const IterArgs& a, bool zero, cudaStream_t s) {
+  if (a.xr.A) return launch_xrow(a, zero ? 2 : 1, s);
   return with_maxr_x(a.maxr_x, [&](auto M) {
     constexpr int MR = decltype(M)::value;
     k_xpass_fwd<MR><<<a.grid_xf * a.nmem, kThreads, xpass_fwd_smem(a), s>>>(a);
@@ -373,7 +373,7 @@ cudaError_t launch_xpass_fwd(const IterArgs& a, cudaStream_t s) {
 }
 
 cudaError_t launch_xpass_inv_fwd(const IterArgs& a, cudaStream_t s) {
-  if (a.xr.A) return launch_xrow(a, false, s);
+  if (a.xr.A) return launch_xrow(a, 0, s);
   return with_maxr_x(a.maxr_x, [&](auto M) {
     constexpr int MR = decltype(M)::value;
     k_xpass_inv_fwd<MR><<<a.grid_x * a.nmem, kThreads, xpass_smem(a), s>>>(a);

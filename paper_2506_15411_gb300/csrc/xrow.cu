@@ -25,8 +25,8 @@ size_t xrow_smem(const IterArgs& a) {
 }
 int xrow_tiles(const IterArgs& a) { return (a.ny * a.nz + a.xr.rpb - 1) / a.xr.rpb; }
 
-cudaError_t launch_xrow(const IterArgs& a, bool first, cudaStream_t s) {
-  row_kernel(a.nx)<<<a.grid_x * a.nmem, 32 * (3 * a.xr.teams + 1), xrow_smem(a), s>>>(a, first ? 1 : 0);
+cudaError_t launch_xrow(const IterArgs& a, int mode, cudaStream_t s) {
+  row_kernel(a.nx)<<<a.grid_x * a.nmem, 32 * (3 * a.xr.teams + 1), xrow_smem(a), s>>>(a, mode);
   return cudaGetLastError();
 }
 

@@ -89,10 +89,10 @@ __device__ __forceinline__ void row_step2(float2* w, int ld, int nr, int lane) {
   }
 }
 
-// The x pass.  first: form V E + S and transform it; else the update pass.  (One kernel: a first
-// pass takes W as 0 and 1 / epsilon as 0, which leaves E as it is.)
+// The x pass.  mode 0: the update pass.  1: form V E + S and transform it (the same code with W
+// and 1 / epsilon taken as 0, which leaves E as it is).  2: the same for E = 0, reading nothing.
 template <int A, int B>
-__global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const int first) {
+__global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const int mode) {
   constexpr int P = row_pitch(B);
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int rpb = a.xr.rpb, S = a.xr.sets, T = a.xr.teams;
@@ -147,18 +147,18 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
         }
         const int r0 = tile * rpb, nr = min(rpb, rows - r0);
         if (lane == 0) {
-          mbar_arrive_expect_tx(full + k, (first ? 4 : 7) * nr * rb);
+          mbar_arrive_expect_tx(full + k, (mode == 0 ? 7 : (mode == 1 ? 4 : 0)) * nr * rb);
           __threadfence_block();
           *issued = ++n;
         }
         __syncwarp();
         float2* const w = set0 + k * set;
         float2* const e = w + 3 * rpb * ldw;
-        for (int i = lane; i < 7 * nr; i += 32) {
+        for (int i = lane; mode < 2 && i < 7 * nr; i += 32) {
           const int arr = ip_div(i, 1.0f / (float)nr), r = i - arr * nr;   // W 0..2, E 3..5, V 6
           const size_t g = (size_t)(r0 + r) * a.nxp;
           if (arr < 3) {
-            if (!first) bulk_load(w + (arr * rpb + r) * ldw, W + arr * a.Nw + g, rb, full + k);
+            if (mode == 0) bulk_load(w + (arr * rpb + r) * ldw, W + arr * a.Nw + g, rb, full + k);
           } else if (arr < 6) {
             bulk_load(e + ((arr - 3) * rpb + r) * lde, E + (arr - 3) * a.Nw + g, rb, full + k);
           } else {
@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
       const int skind = mem.src.kind, splane = skind == 1 ? mem.src.pz : mem.src.zp;
       float2 amp = make_float2(0.f, 0.f);
       if (skind != 2) amp = (skind == 1 && mem.src.amp_dev) ? mem.src.amp_dev[c] : mem.src.amp[c];
-      const float ie = first ? 0.f : mem.inv_eps;
+      const float ie = mode ? 0.f : mem.inv_eps;
       const RowDecode rowdec = row_decode(a);
       float2* const Eg = a.E + so + c * a.Nw;
       float2* const Wg = a.W + so + c * a.Nw;
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
         float2* const w = set0 + k * set + c * rpb * ldw;
         float2* const e = set0 + k * set + 3 * rpb * ldw + c * rpb * lde;
         const float2* const v = set0 + k * set + 3 * rpb * (ldw + lde);
-        if (!first) row_step2<A, B, true>(w, ldw, nr, lane);
+        if (mode == 0) row_step2<A, B, true>(w, ldw, nr, lane);
         constexpr int R = A;
 #pragma unroll 1
         for (int q0 = 0; q0 < nr; q0 += per) {
@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
           float2* const er = e + row * lde + j;
           const float2* const vr = v + row * lde + j;
           float2 x[R];
-          if (!first) {
+          if (mode == 0) {
             x[0] = q[0];
 #pragma unroll
             for (int k1 = 1; k1 < R; ++k1) x[k1] = cmul(q[k1 * P], ip_conj(tw[k1 * B + j]));
@@ -220,6 +220,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
           // E -= delta; then the next iteration's V E
           // (in chunks: the loads of a chunk before its stores)
           constexpr int U = 4;
+          if (mode != 2) {
 #pragma unroll
           for (int r0u = 0; r0u < R; r0u += U) {
             float2 vv[U], ec[U];
@@ -240,6 +241,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
                 acc = fmaf(d.x, d.x, fmaf(d.y, d.y, acc));
                 x[r] = cmul(vv[i2], en);
               }
+          }
           }
           int y, z;
           rowdec(r0 + row, y, z);
@@ -266,7 +268,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
 #pragma unroll
           for (int k1 = 1; k1 < R; ++k1) q[k1 * P] = cmul(x[k1], tw[k1 * B + j]);
         }
-        if (!first) {
+        if (mode == 0) {
           fence_async_smem();
           __syncwarp();
           if (lane == 0) {
@@ -289,7 +291,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
       if (!ok && lane == 0) atomicExch(a.err, kErrTmaTimeout);
     }
   }
-  if (!first) residual_finish(acc, a, mem.seat, mb.b, G, wsum, flags + 1);
+  if (mode == 0) residual_finish(acc, a, mem.seat, mb.b, G, wsum, flags + 1);
   if (lane == 0) bulk_wait_all();
 }
 
