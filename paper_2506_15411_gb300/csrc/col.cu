@@ -22,13 +22,12 @@ size_t col_smem(const ColShape& sh, int ncomp, int twb, int pqb) {
 }  // namespace
 
 cudaError_t launch_col(const CUtensorMap& tm, const IterArgs& a, int kind, cudaStream_t s) {
-  if (kind == colk::kZ) {
-    col_kernels(a.nz).z<<<a.grid_z * a.nmem, a.zc.threads, col_smem(a.zc, 3, a.twbz, a.pqbz), s>>>(tm, a);
-  } else {
-    const ColKernels k = col_kernels(a.ny);
-    (kind == colk::kYFwd ? k.yfwd : k.yinv)<<<a.grid_y * a.nmem, a.yc.threads, col_smem(a.yc, 1, a.twby, 0), s>>>(tm, a);
-  }
-  return cudaGetLastError();
+  if (kind == colk::kZ)
+    return launch_overlapped(col_kernels(a.nz).z, a.grid_z * a.nmem, a.zc.threads,
+                             col_smem(a.zc, 3, a.twbz, a.pqbz), a.N <= kOverlapVoxels, s, tm, a);
+  const ColKernels k = col_kernels(a.ny);
+  return launch_overlapped(kind == colk::kYFwd ? k.yfwd : k.yinv, a.grid_y * a.nmem, a.yc.threads,
+                           col_smem(a.yc, 1, a.twby, 0), a.N <= kOverlapVoxels, s, tm, a);
 }
 
 cudaError_t col_set_smem_limit(int n, bool z, int bytes) {

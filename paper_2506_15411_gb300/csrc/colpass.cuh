@@ -168,6 +168,7 @@ __global__ void __launch_bounds__(col_plan(N, KIND == kZ ? 3 : 1).threads(), 1)
   }
   __syncthreads();
   if (*flags) return;
+  launch_dependents();
 
   const int n = (ntiles - mb.b + G - 1) / G;   // tiles of the block: mb.b, mb.b + G, ...
 
@@ -219,6 +220,7 @@ __global__ void __launch_bounds__(col_plan(N, KIND == kZ ? 3 : 1).threads(), 1)
           tma_load_5d(dst + b * box * TX, &tm, xt * TX, 0, z, b, c0 + c, full + k);
       }
     };
+    wait_for_previous();
     for (int i = 0; i < min(S, n); ++i) load(mb.b + i * G, i);
     if constexpr (!COPY) {
       int k = 0;

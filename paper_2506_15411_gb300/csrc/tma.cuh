@@ -119,6 +119,11 @@ __device__ __forceinline__ void bulk_wait_read_1() {
 // Order this thread's generic-proxy shared-memory writes before later async-proxy reads.
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+// Programmatic dependent launch: let the next kernel of the stream take up processors as this
+// one's blocks leave them, and wait for the kernel before (its writes are then visible).
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Block set-up of a pipelined tile kernel: thread 0 checks that the tile base is 128-byte
 // aligned (as tensor copies require; the tile kernels declare no static shared memory, so the
 // dynamic base is) and initialises the `nbar` mbarriers; a misaligned tile aborts the block

@@ -26,7 +26,10 @@ size_t xrow_smem(const IterArgs& a) {
 int xrow_tiles(const IterArgs& a) { return (a.ny * a.nz + a.xr.rpb - 1) / a.xr.rpb; }
 
 cudaError_t launch_xrow(const IterArgs& a, int mode, cudaStream_t s) {
-  row_kernel(a.nx)<<<a.grid_x * a.nmem, 32 * (3 * a.xr.teams + 1), xrow_smem(a), s>>>(a, mode);
+  const int threads = 32 * (3 * a.xr.teams + 1);
+  if (mode == 0)
+    return launch_overlapped(row_kernel(a.nx), a.grid_x * a.nmem, threads, xrow_smem(a), a.N <= kOverlapVoxels, s, a, 0);
+  row_kernel(a.nx)<<<a.grid_x * a.nmem, threads, xrow_smem(a), s>>>(a, mode);
   return cudaGetLastError();
 }
 

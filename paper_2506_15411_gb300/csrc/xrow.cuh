@@ -128,6 +128,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
     }
     __syncthreads();
     if (flags[0]) return;   // (uniform)
+    launch_dependents();
     const uint32_t rb = (uint32_t)(((a.nx + 1) & ~1) * sizeof(float2));   // bytes of a row copy
     if (warp == 3 * T) {
       // producer: tile i of the block into set i mod S once the tile before it there is done
@@ -138,6 +139,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
         mbar_arrive_expect_tx(tbar, a.twbx);
         bulk_load(tw, a.twx, a.twbx, tbar);
       }
+      wait_for_previous();
       int k = 0, n = 0;
       uint32_t ph = 1;   // a fresh mbarrier passes a wait for the phase before its first
       for (int tile = mb.b; tile < ntiles; tile += G) {
