@@ -193,6 +193,10 @@ int launch_range(cbs_plan_s* p, const IterArgs& a0, int k0, int k1, int m) {
     a.slot = k;
     int rc = launch_iteration(p, a, p->stream, (p->profiling && k == m - 1) ? p->pev : nullptr);
     if (rc) return rc;
+    if (k == k1 - 1 || k % kResidualSlots == kResidualSlots - 1) {
+      const int from = std::max(k0, k / kResidualSlots * kResidualSlots);
+      CK(launch_residuals(a, from, k + 1 - from, 1, p->stream));
+    }
   }
   return CBS_OK;
 }
@@ -391,12 +395,11 @@ void series_begin(cbs_plan_s* p, float2* E, const SourceArgs& src, int warm, Ser
   m.inv_eps = (float)(1.0 / p->eps_s);
   m.kt2 = make_float2((float)p->k0sq_s, (float)p->eps_s);
   m.seat = 0;
-  // every run starts from a clean error flag and residual counter: a run that a timed-out
-  // tensor-copy wait ended left both behind, and everything else it touched (W, the
-  // iterate, the partial sums) is recomputed from the plan's inputs below
+  // every run starts from a clean error flag: a run that a timed-out tensor-copy wait ended left
+  // it behind, and everything else it touched (W, the iterate, the partial sums) is recomputed
+  // from the plan's inputs below
   cudaError_t e = cudaMemcpyAsync(p->mem_dev, p->mem_host, sizeof(Member), cudaMemcpyHostToDevice, p->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(p->Ei, 0, 3 * R.a.Nw * sizeof(float2), p->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(p->counter, 0, sizeof(unsigned), p->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(p->err_dev, 0, sizeof(int), p->stream);
   if (e != cudaSuccess) {
     R.rc = fail(CBS_ERR_CUDA, "field set-up: %s", cudaGetErrorString(e));
@@ -408,6 +411,7 @@ void series_begin(cbs_plan_s* p, float2* E, const SourceArgs& src, int warm, Ser
     a1.slot = 0;
     int rc = launch_xpass_fwd(a1, true, p->stream) == cudaSuccess ? CBS_OK : fail(CBS_ERR_CUDA, "x pass launch failed");
     if (!rc) rc = launch_iteration(p, a1, p->stream, nullptr);
+    if (!rc && launch_residuals(a1, 0, 1, 1, p->stream) != cudaSuccess) rc = fail(CBS_ERR_CUDA, "residual launch failed");
     if (!rc) {
       e = cudaMemcpyAsync(p->hist_host, p->hist, sizeof(double), cudaMemcpyDeviceToHost, p->stream);
       if (e == cudaSuccess) e = cudaMemcpyAsync(p->err_host, p->err_dev, sizeof(int), cudaMemcpyDeviceToHost, p->stream);
@@ -644,7 +648,7 @@ int plan_create(cbs_plan_s** out, const cbs_plan_desc* desc, int seats) {
   // x axes that split into two radices run the warp-per-row passes (xrow.cu)
   CKP(cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device));
   const RowPlan rowp = plan_rows(d.nx, (long long)d.ny * d.nz, p->sms, 226 * 1024,
-                                 (size_t)twb[0] + 8 * 17 + 16 + 32 * 8);
+                                 (size_t)twb[0] + 8 * 17 + 16);
   CKP(rowp.A ? xrow_set_smem_limit(d.nx, 227 * 1024) : xpass_set_smem_limit(227 * 1024));
   a.xr = XRowShape{rowp.A, rowp.B, rowp.ldw, rowp.lde, rowp.rpb, rowp.sets, rowp.teams};
   // y and z tiles: TX columns x whole axis, brought in by boxes of B rows.  B is a divisor of
@@ -751,9 +755,6 @@ int plan_create(cbs_plan_s** out, const cbs_plan_desc* desc, int seats) {
     fail(CBS_ERR_CUDA, "cuTensorMapEncodeTiled failed for the workspace");
     return bail(CBS_ERR_CUDA);
   }
-  CKP(cudaMalloc(&p->partials, S * std::max(xpass_tiles(a), a.xr.A ? xrow_tiles(a) : 0) * sizeof(double)));   // >= seats x the x grid
-  CKP(cudaMalloc(&p->counter, S * sizeof(unsigned)));
-  CKP(cudaMemset(p->counter, 0, S * sizeof(unsigned)));
   CKP(cudaMalloc(&p->hist, S * d.check_every * sizeof(double)));
   CKP(cudaMallocHost(&p->hist_host, S * d.check_every * sizeof(double)));
   CKP(cudaMalloc(&p->mem_dev, members_len(seats, d.check_every) * sizeof(Member)));
@@ -828,6 +829,7 @@ int plan_create(cbs_plan_s** out, const cbs_plan_desc* desc, int seats) {
   {
     CKP(x_grid_size(a, p->sms));
     CKP(yz_grid_sizes(a, p->sms));
+    CKP(cudaMalloc(&p->partials, S * kResidualSlots * a.grid_x * sizeof(double)));
   }
 
   // every address the tile kernels bulk-copy from or to must be 16-byte aligned, every size
@@ -862,7 +864,6 @@ int plan_create(cbs_plan_s** out, const cbs_plan_desc* desc, int seats) {
   a.mem = p->mem_dev;
   a.err = p->err_dev;
   a.partials = p->partials;
-  a.counter = p->counter;
   a.hist = p->hist;
   a.hist_cap = d.check_every;
   a.invN = (float)(1.0 / (double)N);
@@ -885,7 +886,7 @@ void cbs_destroy(cbs_plan_t p) {
   cudaSetDevice(p->device);
   if (p->stream) cudaStreamSynchronize(p->stream);
   drop_graphs(p);
-  void* devs[] = {p->V, p->W, p->Ei, p->tw, p->pq, p->stages, p->partials, p->counter, p->hist, p->mem_dev,
+  void* devs[] = {p->V, p->W, p->Ei, p->tw, p->pq, p->stages, p->partials, p->hist, p->mem_dev,
                   p->adj_amp, p->dobj,
                   p->sx, p->sy, p->sz, p->pmin, p->pmax, p->pbad, p->pdev, p->split, p->eps_dev,
                   p->Ef, p->Ea, p->grad_dev, p->err_dev};

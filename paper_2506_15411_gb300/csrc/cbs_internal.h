@@ -28,6 +28,7 @@ struct SourceArgs {
 // block b mod grid of that request's own persistent grid, so every request's tiles, and the
 // order of its residual sums, are the same in any launch.
 constexpr int kMaxMembers = 8;
+constexpr int kResidualSlots = 64;   // iterations whose residual partials are kept
 
 struct Member {
   SourceArgs src;
@@ -100,8 +101,7 @@ struct IterArgs {
   int nmem;               // members of this launch (1 .. kMaxMembers)
   const Member* mem;      // their sources, splittings and seats (device memory)
   float invN;             // 1 / N, folded into the k-space multiply
-  double* partials;       // residual partial sums, [seat][grid_x]
-  unsigned* counter;      // last-block-done counters, [seat] (left at 0)
+  double* partials;       // residual partial sums, [seat][kResidualSlots][grid_x]
   double* hist;           // hist[seat * hist_cap + slot] = sum |delta|^2 of this iteration
   int hist_cap;
   int slot;
@@ -144,6 +144,10 @@ cudaError_t launch_xpass_fwd(const IterArgs& a, bool zero, cudaStream_t s);   //
 cudaError_t launch_ypass(const CUtensorMap& tm, const IterArgs& a, bool inverse, cudaStream_t s);
 cudaError_t launch_zpass_green(const CUtensorMap& tm, const IterArgs& a, cudaStream_t s);  // FFTz, G, IFFTz
 cudaError_t launch_xpass_inv_fwd(const IterArgs& a, cudaStream_t s);  // IFFTx, update, residual, next FFTx
+
+// Sum the residual partials of iterations slot0 .. slot0 + count - 1 (count <= kResidualSlots, none of
+// them wrapped) of seats 0 .. seats - 1 into hist.
+cudaError_t launch_residuals(const IterArgs& a, int slot0, int count, int seats, cudaStream_t s);
 
 // Shared-memory bytes and threads of each pass for the plan's shapes.
 size_t xpass_smem(const IterArgs& a);

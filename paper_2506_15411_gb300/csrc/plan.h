@@ -84,7 +84,6 @@ struct cbs_plan_s {
   int4* stages = nullptr;
   std::vector<int> radix_order[3];  // DIF radix order of each axis
   double* partials = nullptr;
-  unsigned* counter = nullptr;
   double* hist = nullptr;
   cbs::Member* mem_dev = nullptr;   // launch members (members_len) and their pinned staging
   cbs::Member* mem_host = nullptr;

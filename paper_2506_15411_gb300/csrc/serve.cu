@@ -245,7 +245,7 @@ int make_batch(cbs_server_s* S, const ShapeKey& k, int seats, Batch** out) {
 }
 
 // Start the series of seat s (field `E` receives the result) with source `src`: the seat's
-// iterate and residual counter are cleared and the series' first x pass is enqueued on the
+// iterate is cleared and the series' first x pass is enqueued on the
 // batch's stream, after whatever is in flight there; the seat takes part from the next block.
 int seat_begin(Batch* b, Seat& s, float2* E, const SourceArgs& src, Phase phase) {
   cbs_plan_s* p = b->plan;
@@ -256,7 +256,6 @@ int seat_begin(Batch* b, Seat& s, float2* E, const SourceArgs& src, Phase phase)
   s.blk = 0;
   const size_t Nw = p->base.Nw;
   CK(cudaMemsetAsync(p->Ei + (size_t)s.idx * 3 * Nw, 0, 3 * Nw * sizeof(float2), b->stream));
-  CK(cudaMemsetAsync(p->counter + s.idx, 0, sizeof(unsigned), b->stream));
   // the seat's own member slot (its previous copy completed with its previous series)
   p->mem_host[1 + s.idx] = s.mem;
   CK(cudaMemcpyAsync(p->mem_dev + 1 + s.idx, p->mem_host + 1 + s.idx, sizeof(Member), cudaMemcpyHostToDevice,
@@ -346,6 +345,10 @@ int enqueue_block(cbs_server_s* S, Batch* b) {
     a.slot = k;
     const int rc = launch_iteration(p, a, b->stream, nullptr);
     if (rc) return rc;
+    if (k == L - 1 || k % kResidualSlots == kResidualSlots - 1) {
+      const int from = k / kResidualSlots * kResidualSlots;
+      CK(launch_residuals(a, from, k + 1 - from, p->seats, b->stream));
+    }
     std::lock_guard<std::mutex> lk(S->mu);
     S->n_launches += 1;
     S->n_member_iters += a.nmem;

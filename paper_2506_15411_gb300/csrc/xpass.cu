@@ -63,7 +63,6 @@ struct XTile {
   uint64_t* full;   // [nset]
   uint64_t* tbar;   // the twiddle table's copy
   int* fail;        // [2]: per warp group
-  int* last;
   double* wsum;
 };
 
@@ -79,7 +78,6 @@ __device__ __forceinline__ XTile carve(unsigned char* base, int rpb, int nxp, in
   t.full = reinterpret_cast<uint64_t*>(p);
   t.tbar = t.full + nset;
   t.fail = reinterpret_cast<int*>(t.tbar + 1);
-  t.last = t.fail + 2;
   t.wsum = reinterpret_cast<double*>(t.fail + 4);
   return t;
 }
@@ -319,7 +317,7 @@ __global__ void __launch_bounds__(kThreads, kXOcc) k_xpass_inv_fwd(const IterArg
       }
     }
   }
-  residual_finish(acc, a, mem.seat, mb.b, G, t.wsum, t.last);
+  residual_finish(acc, a, mem.seat, mb.b, t.wsum);
   if (lt == 0) bulk_wait_all();
 }
 
@@ -334,6 +332,26 @@ size_t xpass_fwd_smem(const IterArgs& a) {
   return (size_t)4 * a.nset_xf * a.rpb * a.nxp * sizeof(float2) + a.twbx + 8 * (a.nset_xf + 1) + 16 + 32 * 8;
 }
 int xpass_tiles(const IterArgs& a) { return (a.ny * a.nz + a.rpb - 1) / a.rpb; }
+
+namespace {
+
+// hist[slot0 + i] of each seat: the sum of that iteration's block partials.
+__global__ void k_residuals(const IterArgs a, int slot0) {
+  const int slot = slot0 + blockIdx.x, seat = blockIdx.y, lane = threadIdx.x;
+  const double* const part = a.partials + ((size_t)seat * kResidualSlots + slot % kResidualSlots) * a.grid_x;
+  double s = 0.0;
+  for (int b = lane; b < a.grid_x; b += 32) s += part[b];
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+  if (lane == 0) a.hist[(size_t)seat * a.hist_cap + slot] = s;
+}
+
+}  // namespace
+
+cudaError_t launch_residuals(const IterArgs& a, int slot0, int count, int seats, cudaStream_t s) {
+  k_residuals<<<dim3(count, seats), 32, 0, s>>>(a, slot0);
+  return cudaGetLastError();
+}
 
 template <class F>
 cudaError_t with_maxr_x(int maxr, F&& f) {

@@ -21,13 +21,16 @@ __device__ __forceinline__ RowDecode row_decode(const IterArgs& a) {
   return RowDecode{1.0f / (float)a.yblk, 1.0f / (float)a.nz, a.yblk, a.nz};
 }
 
-// Block reduction of the per-thread residual in FP64, then a last-block-done pass that sums
-// the per-block partials of the request in seat `seat` (blocks b = 0 .. G-1 of its grid) in a
-// fixed order into its hist[slot] (deterministic).
-__device__ __forceinline__ void residual_finish(float acc, const IterArgs& a, int seat, int b, int G, double* wsum,
-                                                int* lastflag) {
-  double* const part = a.partials + (size_t)seat * a.grid_x;
-  unsigned* const counter = a.counter + seat;
+// Where block b of a request's grid leaves its residual partial of the current iteration: the
+// partials of kResidualSlots iterations are kept, and k_residuals sums each iteration's in a fixed
+// order once per that many (or at the end of a block of iterations).  A last-block-done sum in the
+// x pass itself would add two trips through memory to every iteration.
+__device__ __forceinline__ double* residual_slot(const IterArgs& a, int seat, int b) {
+  return a.partials + ((size_t)seat * kResidualSlots + a.slot % kResidualSlots) * a.grid_x + b;
+}
+
+// Block sum of the per-thread residual in FP64 (fixed order) into the block's slot.
+__device__ __forceinline__ void residual_finish(float acc, const IterArgs& a, int seat, int b, double* wsum) {
   double d = (double)acc;
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) d += __shfl_down_sync(0xffffffffu, d, off);
@@ -38,26 +41,7 @@ __device__ __forceinline__ void residual_finish(float acc, const IterArgs& a, in
   if (threadIdx.x == 0) {
     double bs = 0.0;
     for (int w = 0; w < nw; ++w) bs += wsum[w];
-    part[b] = bs;
-    __threadfence();
-    const unsigned prev = atomicAdd(counter, 1u);
-    *lastflag = (prev == (unsigned)G - 1);
-  }
-  __syncthreads();
-  if (!*lastflag) return;
-  __threadfence();
-  double s = 0.0;
-  for (int i = threadIdx.x; i < G; i += blockDim.x) s += __ldcg(&part[i]);
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-  __syncthreads();
-  if (lane == 0) wsum[wid] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double bs = 0.0;
-    for (int w = 0; w < nw; ++w) bs += wsum[w];
-    a.hist[(size_t)seat * a.hist_cap + a.slot] = bs;
-    *counter = 0u;
+    *residual_slot(a, seat, b) = bs;
   }
 }
 

@@ -18,10 +18,11 @@ RowKernel row_kernel(int n) {
 }  // namespace
 
 // S sets of rpb rows (W of three components at pitch ldw, E of three and V at pitch lde), the
-// twiddles, 2 S + 1 mbarriers, the flags and the warps' sums
+// twiddles, 2 S + 1 mbarriers and the flags
 size_t xrow_smem(const IterArgs& a) {
-  return (size_t)a.xr.sets * a.xr.rpb * (3 * a.xr.ldw + 4 * a.xr.lde) * sizeof(float2) + a.twbx +
-         8 * (2 * a.xr.sets + 1) + 16 + 32 * 8;
+  const size_t sets = (size_t)a.xr.sets * a.xr.rpb * (3 * a.xr.ldw + 4 * a.xr.lde) * sizeof(float2) + a.twbx +
+                      8 * (2 * a.xr.sets + 1) + 16;
+  return std::max(sets, (size_t)xrow::kRowThreads * sizeof(float));   // (at the end: the threads' residuals)
 }
 int xrow_tiles(const IterArgs& a) { return (a.ny * a.nz + a.xr.rpb - 1) / a.xr.rpb; }
 

@@ -105,9 +105,8 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
   uint64_t* const full = reinterpret_cast<uint64_t*>(tw + a.twbx / sizeof(float2));   // [S]
   uint64_t* const empty = full + S;                                                   // [S]
   uint64_t* const tbar = empty + S;
-  int* const flags = reinterpret_cast<int*>(tbar + 1);   // alignment failure, last block
-  volatile int* const issued = flags + 2;                // tiles of the block issued so far
-  double* const wsum = reinterpret_cast<double*>(flags + 4);
+  int* const flags = reinterpret_cast<int*>(tbar + 1);   // alignment failure
+  volatile int* const issued = flags + 1;                // tiles of the block issued so far
 
   const MemberBlock mb = member_block(blockIdx.x, G);
   const Member& mem = a.mem[mb.j];
@@ -293,7 +292,21 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
       if (!ok && lane == 0) atomicExch(a.err, kErrTmaTimeout);
     }
   }
-  if (mode == 0) residual_finish(acc, a, mem.seat, mb.b, G, wsum, flags + 1);
+  if (mode == 0) {
+    // the block's residual: the threads' sums through shared memory (every tile has been read out
+    // of it by now), one warp adds them in FP64 in a fixed order
+    float* const sums = reinterpret_cast<float*>(smem_raw);
+    __syncthreads();
+    sums[tid] = acc;
+    __syncthreads();
+    if (warp == 0) {
+      double d = 0.0;
+      for (int i = lane; i < blockDim.x; i += 32) d += (double)sums[i];
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) d += __shfl_down_sync(0xffffffffu, d, off);
+      if (lane == 0) *residual_slot(a, mem.seat, mb.b) = d;
+    }
+  }
   if (lane == 0) bulk_wait_all();
 }
 
