@@ -71,13 +71,19 @@ __device__ __forceinline__ void col_step1(float2* buf, int cs, const float2* tw,
     for (int r = 0; r < A; ++r) v[r] = (INV && SW && (r & 1) ? odd : even)[r * B * TX];
     if constexpr (INV) {
 #pragma unroll
-      for (int r = 1; r < A; ++r) v[r] = cmul(v[r], ip_conj(w[r * B]));
+      for (int r = 1; r < A; ++r) {
+        v[r] = cmul(v[r], ip_conj(w[r * B]));
+        if (r % 8 == 0) asm volatile("" ::: "memory");   // (keeps the twiddles of a few products in registers, not all)
+      }
     }
     DFT<A, INV>::run(v);
     if constexpr (SW) __syncwarp();
     if constexpr (!INV) {
 #pragma unroll
-      for (int r = 1; r < A; ++r) v[r] = cmul(v[r], w[r * B]);
+      for (int r = 1; r < A; ++r) {
+        v[r] = cmul(v[r], w[r * B]);
+        if (r % 8 == 0) asm volatile("" ::: "memory");
+      }
     }
     if (on) {
 #pragma unroll
