@@ -209,16 +209,17 @@ constexpr int row_pitch(int B) { return B + (6 - B % 4) % 4; }   // least pitch 
 
 // Modelled work of a tile of rpb rows, whole rounds of 32 / B and 32 / A rows counted: step 1
 // (radix A) runs both transforms, the update and two twiddle products; step 2 (radix B) runs once
-// forward and once inverse, and a long one is dear: it holds B values between two warp barriers
-// and moves them as 16-byte pairs (640 on one plane of rows: 32 x 20 2.13 ms, 20 x 32 3.48 ms;
-// 275: 25 x 11 0.44 ms, 11 x 25 0.63 ms).
+// forward and once inverse, and counts half more from 30 values on, which it moves as 16-byte pairs
+// between two warp barriers.  Measured (rows of 64 x 64 grids, us): 400 as 16 x 25 32.7, 20 x 20 37.2,
+// 25 x 16 41.1; 275 as 11 x 25 27.2, 25 x 11 30.4; 512 as 16 x 32 39.1, 32 x 16 45.1; 256 as 16 x 16 22.5, 8 x 32
+// 22.5, 32 x 8 28.7; 640 x 640 x 336, where memory decides: 32 x 20 2.14 ms, 20 x 32 2.28 ms.
 constexpr int row_tile_cost(int A, int B, int rpb) {
   const int per1 = 32 / B, per2 = 32 / A;
   const int w1 = A * (2 * radix_cost(A) + 36), w2 = 2 * B * (radix_cost(B) + 2);
-  return (rpb + per1 - 1) / per1 * w1 + (rpb + per2 - 1) / per2 * (B > 16 ? w2 * 5 / 2 : w2);
+  return (rpb + per1 - 1) / per1 * w1 + (rpb + per2 - 1) / per2 * (B >= 30 ? w2 * 3 / 2 : w2);
 }
 
-// The larger radix A of the split n = A B an axis' kernels are built for (0: none): the least
+// The radix A of step 1 of the split n = A B an axis' kernels are built for (0: none): the least
 // work per row over tiles of 1, 2 and 4 rows that leave room for six of them (a row of an axis
 // too long for that is taken alone).
 constexpr int row_split(int n) {
