@@ -400,8 +400,10 @@ def run_gpu(args, rank, world, local_rank):
         for _ in range(args.steps):
             sf, sa, obj = step()
             iters += sf.iters + sa.iters
-            # set-up 3 + forward (1 + 4/iter) + adjoint source 1 + adjoint (1 + 4/iter) + gradient 2
-            launches += 3 + 1 + 4 * sf.iters + 1 + 1 + 4 * sa.iters + 2
+            # set-up 3 + forward (1 + 4/iter) + adjoint source 1 + adjoint (1 + 4/iter) + gradient 2,
+            # and one sum of the residuals per block of iterations and 64 of them
+            sums = sum(-(-st.iters // check) * -(-check // 64) for st in (sf, sa))
+            launches += 3 + 1 + 4 * sf.iters + 1 + 1 + 4 * sa.iters + 2 + sums
             stats.append((sf, sa, obj))
         ev1.record(stream)
         barrier()

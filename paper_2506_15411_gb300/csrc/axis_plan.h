@@ -369,8 +369,8 @@ inline RowPlan plan_rows(int n, long long rows, int sms, size_t budget, size_t f
   // rows of a tile and teams: the least work of the busiest processor (its tiles times a tile's
   // work and a tile's fixed part), with a set per team and one in flight unless a single row is
   // too long for that.  Four teams where only they leave room for the better-filled rounds
-  // (384 = 24 x 16: two rows 0.665 ms, one row with five teams 0.771 ms), and one team less when
-  // the sets just suffice for single rows (640: 2.14 against 2.20 ms).
+  // (384 as 24 x 16: two rows 0.665 ms, one row with five teams 0.771 ms; as 16 x 24 0.62), and one
+  // team less when the sets just suffice for single rows (640: 2.14 against 2.20 ms).
   double least = 1e300;
   for (int teams : {5, 4})
     for (int rpb = 1; rpb <= 32; ++rpb) {

@@ -25,7 +25,7 @@
 // copy), 384 x 384 x 256 0.290 -> 0.290, 175 x 175 x 198 0.070 -> 0.050, 104 x 104 x 120 (a factor
 // 13) 0.039 -> 0.0165, 128^3 0.030 -> 0.019.  z, also 48 bytes, by instruction issue and shared
 // memory, about half of each busy: 640 x 640 x 336 1.88 -> 1.36 (0.71 of a copy), 384 x 384 x 256
-// 0.616 -> 0.334 (0.80), 275 x 275 x 315 0.371 -> 0.309, 256 x 256 x 192 0.165 -> 0.111 (0.80),
+// 0.616 -> 0.338 (0.79), 275 x 275 x 315 0.371 -> 0.302, 256 x 256 x 192 0.165 -> 0.111 (0.80),
 // 128^3 0.045 -> 0.025.  The staged passes took three to four stages each way, a barrier and a
 // trip through shared memory each, with offsets computed at run time.
 #pragma once

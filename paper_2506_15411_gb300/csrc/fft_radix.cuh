@@ -1,9 +1,10 @@
 // fft_radix.cuh -- small in-register DFTs ("codelets") for the mixed-radix FFT passes.
 //
 // The 3D FFTs of the CBS iteration (the "N log N" cost of Fig. 1(b) of arXiv 2506.15411)
-// are built from in-place DIF / DIT stages (fft_ip.cuh) whose butterflies are the DFTs below, applied to R values
-// held in registers.  Supported radices: 1 (identity) to 13 and 16, and for the kernels that
-// transform an axis in two steps also 14, 15, 18, 20, 21, 22, 24 to 28, 30, 32, 35 and 36.
+// are built from the DFTs below, applied to R values held in registers: two steps of compile-time
+// radices (xrow.cuh, colpass.cuh), or in-place DIF / DIT stages (fft_ip.cuh) of 1 (identity) to 13
+// and 16 for axes that do not split so.  The two steps also use 14, 15, 18, 20, 21, 22, 24 to 28,
+// 30, 32, 35 and 36.
 //   - odd primes: symmetric-pair form, X[k] and X[R-k] share the sums over the pairs
 //     x[m] +- x[R-m] with real cos/sin constants;
 //   - composites: one Cooley-Tukey split R = R1 * R2 (decimation in time) with the inner
@@ -240,8 +241,8 @@ template <bool INV> struct DFT<35, INV> : DFTSplit<5, 7, INV> {};
 template <bool INV> struct DFT<36, INV> : DFTSplit<4, 9, INV> {};
 
 // Calls f(std::integral_constant<int, R>) for the runtime radix r (uniform across the block).
-// Radices above MAXR are not compiled in (a plan whose axes need them uses a MAXR = 16
-// kernel); leaving them out keeps the register allocation to what the smaller radices need.
+// The stages' radices: 1 to 13 and 16.  Those above MAXR are not compiled in (a plan whose axes
+// need them uses a MAXR = 16 kernel); leaving them out keeps the register allocation to what the smaller radices need.
 template <int MAXR = 16, class F>
 CBS_HD void radix_dispatch(int r, F&& f) {
   switch (r) {
@@ -258,22 +259,7 @@ CBS_HD void radix_dispatch(int r, F&& f) {
     case 11: if constexpr (MAXR >= 11) f(std::integral_constant<int, 11>{}); break;
     case 12: if constexpr (MAXR >= 12) f(std::integral_constant<int, 12>{}); break;
     case 13: if constexpr (MAXR >= 13) f(std::integral_constant<int, 13>{}); break;
-    case 14: if constexpr (MAXR > 16) f(std::integral_constant<int, 14>{}); break;
-    case 15: if constexpr (MAXR > 16) f(std::integral_constant<int, 15>{}); break;
     case 16: if constexpr (MAXR >= 16) f(std::integral_constant<int, 16>{}); break;
-    case 18: if constexpr (MAXR >= 18) f(std::integral_constant<int, 18>{}); break;
-    case 20: if constexpr (MAXR >= 20) f(std::integral_constant<int, 20>{}); break;
-    case 21: if constexpr (MAXR >= 21) f(std::integral_constant<int, 21>{}); break;
-    case 22: if constexpr (MAXR >= 22) f(std::integral_constant<int, 22>{}); break;
-    case 24: if constexpr (MAXR >= 24) f(std::integral_constant<int, 24>{}); break;
-    case 25: if constexpr (MAXR >= 25) f(std::integral_constant<int, 25>{}); break;
-    case 26: if constexpr (MAXR >= 26) f(std::integral_constant<int, 26>{}); break;
-    case 27: if constexpr (MAXR >= 27) f(std::integral_constant<int, 27>{}); break;
-    case 28: if constexpr (MAXR >= 28) f(std::integral_constant<int, 28>{}); break;
-    case 30: if constexpr (MAXR >= 30) f(std::integral_constant<int, 30>{}); break;
-    case 32: if constexpr (MAXR >= 32) f(std::integral_constant<int, 32>{}); break;
-    case 35: if constexpr (MAXR >= 35) f(std::integral_constant<int, 35>{}); break;
-    case 36: if constexpr (MAXR >= 36) f(std::integral_constant<int, 36>{}); break;
     default: break;
   }
 }

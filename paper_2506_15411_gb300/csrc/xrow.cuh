@@ -23,9 +23,10 @@
 // Bound by memory: 104 bytes a voxel.  The staged pass (xpass.cu) spent its time at barriers and
 // on shared memory, which its three or four stages cross 17 times per value, and on their bank
 // conflicts; this one crosses it 13 times without.  Update pass, staged -> rows (ms, one GB300):
-// 640 x 640 x 336 2.91 -> 2.14 (6.7 TB/s, 0.99 of a copy), 384 x 384 x 256 0.966 -> 0.625 (0.93),
-// 275 x 275 x 315 0.649 -> 0.436 (0.84; 22 and 25 of 32 lanes hold values), 256 x 256 x 192 0.356
-// -> 0.221, 175 x 175 x 198 0.163 -> 0.119, 128^3 0.076 -> 0.049; 64^3 0.0214 -> 0.0205 (latency).
+// 640 x 640 x 336 2.91 -> 2.16 (6.6 TB/s, 0.97 of a copy), 384 x 384 x 256 0.966 -> 0.62 (0.93),
+// 275 x 275 x 315 0.649 -> 0.386 (0.95), 256 x 256 x 192 0.356 -> 0.219 (0.88), 175 x 175 x 198
+// 0.163 -> 0.108 (0.86), 192 x 192 x 128 0.128 -> 0.084 (0.86), 128^3 0.076 -> 0.047; 64^3 0.0214
+// -> 0.0184 (latency of one to three tiles a block).
 #pragma once
 #include <algorithm>
 
