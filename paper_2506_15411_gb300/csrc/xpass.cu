@@ -1,4 +1,5 @@
-// xpass.cu -- the passes along x (contiguous rows) of the CBS iterations.
+// xpass.cu -- the passes along x (contiguous rows) of the CBS iterations, for axes that do not
+// split into two radices (others: xrow.cuh), the choice between the two, and the residual sums.
 //
 //   forward:  W_c = FFT_x(V E_c + S_c)                       (scattering potential and source
 //                                                              formed as the first FFT stage

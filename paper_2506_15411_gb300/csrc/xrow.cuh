@@ -22,7 +22,8 @@
 //
 // Bound by memory: 104 bytes a voxel.  The staged pass (xpass.cu) spent its time at barriers and
 // on shared memory, which its three or four stages cross 17 times per value, and on their bank
-// conflicts; this one crosses it 13 times without.  Update pass, staged -> rows (ms, one GB300):
+// conflicts; this one crosses it 13 times with two fifths of the conflicts (275 x 275 x 315: 47 ->
+// 19 million; a quarter on rows of 640).  Update pass, staged -> rows (ms, one GB300):
 // 640 x 640 x 336 2.91 -> 2.16 (6.6 TB/s, 0.97 of a copy), 384 x 384 x 256 0.966 -> 0.62 (0.93),
 // 275 x 275 x 315 0.649 -> 0.386 (0.95), 256 x 256 x 192 0.356 -> 0.219 (0.88), 175 x 175 x 198
 // 0.163 -> 0.108 (0.86), 192 x 192 x 128 0.128 -> 0.084 (0.86), 128^3 0.076 -> 0.047; 64^3 0.0214

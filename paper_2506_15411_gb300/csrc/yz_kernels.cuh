@@ -1,4 +1,5 @@
-// yz_kernels.cuh -- the strided passes of one CBS iteration, fed by the Tensor Memory Accelerator.
+// yz_kernels.cuh -- the strided passes of one CBS iteration, fed by the Tensor Memory Accelerator,
+// for axes that colpass.cuh has no two-step kernel for.
 //
 //   y pass:  W_c <- FFT_y(W_c) or IFFT_y(W_c), one (component, z) plane x TX columns per tile
 //   z pass:  W <- IFFT_z( G(p) FFT_z(W) ), the three components of one y row x TX columns,

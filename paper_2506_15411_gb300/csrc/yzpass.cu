@@ -1,6 +1,6 @@
 // yzpass.cu -- host side of the strided passes (y, and z with the k-space multiply): launch
-// shapes, grid sizes and launches.  The kernels are in yz_kernels.cuh and are compiled per
-// tile width in ypass_tx*.cu / zpass_tx*.cu.
+// shapes, grid sizes and launches.  The kernels are in yz_kernels.cuh, compiled per tile width in
+// ypass_tx*.cu / zpass_tx*.cu; axes with a two-step split go to colpass.cuh's (col.cu).
 #include <algorithm>
 
 #include "yz_kernels.cuh"
