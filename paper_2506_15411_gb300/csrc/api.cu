@@ -292,6 +292,10 @@ cudaError_t field_copy(const cbs_plan_s* p, int seat, float2* dense, bool to_den
 // and the event the host waits on.
 int series_enqueue_block(cbs_plan_s* p, SeriesRun& R) {
   R.m = std::min(p->d.check_every, p->d.max_iter - R.it);
+  if (p->mem_host[0].phase != R.it % kTwiddlePhases) {   // (its last copy completed with the last block)
+    p->mem_host[0].phase = R.it % kTwiddlePhases;
+    CK(cudaMemcpyAsync(p->mem_dev, p->mem_host, sizeof(Member), cudaMemcpyHostToDevice, p->stream));
+  }
   R.blk_range = nvtxRangeStartA("cbs: block of iterations");
   // full blocks replay a graph; with profiling the last iteration runs outside it
   const int ng = (R.m == p->d.check_every) ? (p->profiling ? R.m - 1 : R.m) : 0;
@@ -738,6 +742,9 @@ int plan_create(cbs_plan_s** out, const cbs_plan_desc* desc, int seats) {
   a.twbx = twb[0];
   a.twby = twb[1];
   a.twbz = twb[2];
+  a.twsx = rowp.A ? twiddle_stride(d.nx) : 0;
+  a.twsy = yp.A ? twiddle_stride(d.ny) : 0;
+  a.twsz = zp.A ? twiddle_stride(d.nz) : 0;
   a.pqbz = pqbz;
 
   const size_t N = p->N;
@@ -777,8 +784,8 @@ int plan_create(cbs_plan_s** out, const cbs_plan_desc* desc, int seats) {
 
   // per-axis FFT tables (axis_plan.h): radix order for the axis' shared-memory layout, stage
   // table, per-stage twiddles (FP64, rounded; padded to n entries so that a fixed n * 8 bytes
-  // are copied into the tiles) and the wave numbers of each spectrum position (padded to 16
-  // entries); every table starts on a 128-byte boundary
+  // are copied into the tiles) and the wave numbers (p^2, q) of each spectrum position (padded
+  // to 16 entries); every table starts on a 128-byte boundary
   {
     const AxisLayout lay[3] = {AxisLayout::Rows, AxisLayout::Cols, AxisLayout::ColsZ};
     const int ncol[3] = {0, a.tx_y, a.tx_z};
@@ -797,9 +804,10 @@ int plan_create(cbs_plan_s** out, const cbs_plan_desc* desc, int seats) {
       if (a2 == 0 && rowp.A) row_tables(n, rowp, tw, pq);
       if (a2 == 1 && yp.A) col_tables(n, yp, true, tw, pq);
       if (a2 == 2 && zp.A) col_tables(n, zp, false, tw, pq);
+      square_wave_numbers(n, pq);
       std::copy(st.begin(), st.end(), st_all.begin() + a2 * 2 * kMaxAxisStages);
       twoff[a2] = (int)tw_all.size();
-      tw.resize(round_up(n, 16), make_float2(0.f, 0.f));
+      tw.resize(round_up(std::max(n, (int)tw.size()), 16), make_float2(0.f, 0.f));
       tw_all.insert(tw_all.end(), tw.begin(), tw.end());
       pqoff[a2] = (int)pq_all.size();
       pq.resize(round_up(n, 16), make_float2(0.f, 0.f));
@@ -867,6 +875,7 @@ int plan_create(cbs_plan_s** out, const cbs_plan_desc* desc, int seats) {
   a.hist = p->hist;
   a.hist_cap = d.check_every;
   a.invN = (float)(1.0 / (double)N);
+  a.invN_rest = (float)((1.0 / (double)N - (double)a.invN) / (double)a.invN);
 #undef CKP
   *out = p;
   return CBS_OK;

@@ -12,7 +12,15 @@
 #include <functional>
 #include <vector>
 
+#include "fft_radix.cuh"   // unit_pair
+
 namespace cbs {
+
+// exp(i a) as a table entry
+inline float2 unit_twiddle(double a) {
+  const CosSin w = unit_pair(std::cos(a), std::sin(a));
+  return make_float2(w.c, w.s);
+}
 
 constexpr int kMaxAxisStages = 8;
 
@@ -190,9 +198,36 @@ inline std::vector<int> order_radices_z(const std::vector<int>& radices, int n, 
   return best;
 }
 
+// ------------------------------------------------------------- twiddles of the two-step passes
+// kTwiddlePhases tables one after the other, `stride` values apart, each used by every
+// kTwiddlePhases-th iteration: a value's roundings carry their error on from one table to the
+// next, so that over the cycle they average to the value to a fraction of a rounding.  One rounded
+// table's errors would act in the same direction in every iteration: they were half of the
+// gradient's error (65 x 56 x 48: 2.4 -> 0.7e-6).
+constexpr int twiddle_stride(int n) { return (n + 15) / 16 * 16; }
+
+// Twiddles w_n^{j k1} at k1 B + j, j < B = n / A, of every phase.
+inline void phased_twiddles(int n, int A, std::vector<float2>& tw) {
+  const double two_pi = 6.283185307179586476925287;
+  const int B = n / A, stride = twiddle_stride(n);
+  tw.assign((size_t)kTwiddlePhases * stride, make_float2(0.f, 0.f));
+  for (int k = 0; k < A; ++k)
+    for (int j = 0; j < B; ++j) {
+      const double a = -two_pi * (double)((long long)j * k % n) / (double)n, c = std::cos(a), s = std::sin(a);
+      double cc = 0.0, ss = 0.0;   // carried
+      for (int f = 0; f < kTwiddlePhases; ++f) {
+        const float2 w = make_float2((float)(c + cc), (float)(s + ss));
+        cc += c - (double)w.x;
+        ss += s - (double)w.y;
+        tw[(size_t)f * stride + k * B + j] = w;
+      }
+    }
+}
+
 // --------------------------------------------------------------- x rows in two steps (xrow.cuh)
 // Instructions per value of a radix' in-register transform, roughly: what its split costs (the
-// odd primes' symmetric sums, one constant twiddle per value of a split).
+// odd primes' symmetric sums, one constant twiddle per value of a split; coprime splits have none,
+// but count as the others, as the plans were measured so).
 constexpr int radix_cost(int R) {
   if (R <= 2) return R - 1;
   if (R == 4) return 2;
@@ -252,7 +287,9 @@ constexpr int z_box_rows(int n, int tx) {
   return tx == 8 ? (rows + 1) / 2 * 2 : rows;
 }
 // Shared memory of a block but its tiles: twiddles, wave numbers (z), mbarriers and flags.
-constexpr int col_fixed_smem(int n, int ncomp) { return (n + 1) / 2 * 16 * (ncomp == 3 ? 2 : 1) + 8 * 17 + 48; }
+constexpr int col_fixed_smem(int n, int ncomp) {
+  return (n + 1) / 2 * 16 * (ncomp == 3 ? 2 : 1) + 8 * 17 + 48;
+}
 constexpr int kColSmem = 226 * 1024;
 
 // Shape of the y (ncomp = 1) or z (3) kernels of an axis of n; A = 0: none.  Radices up to 32 (z:
@@ -304,17 +341,21 @@ constexpr ColPlan col_plan(int n, int ncomp) {
   return best;
 }
 
+// (p, q) of an axis' table to (p^2, q), the squares from FP64 (a frequency's p is 2 pi k / n).
+inline void square_wave_numbers(int n, std::vector<float2>& pq) {
+  const double step = 6.283185307179586476925287 / (double)n;
+  for (float2& e : pq) {
+    const double p = std::round((double)e.x / step) * step;
+    e.x = (float)(p * p);
+  }
+}
+
 // Tables of a column axis: twiddles w_n^{j k1} at k1 B + j; wave numbers by row (y: frequency
 // k1 + A k2 sits in row k1 B + (k2 ^ s), s = k1 & 1 for 8 columns and even B) or by frequency (z).
 inline void col_tables(int n, const ColPlan& p, bool by_row, std::vector<float2>& tw, std::vector<float2>& pq) {
   const double two_pi = 6.283185307179586476925287;
   const int A = p.A, B = n / A;
-  tw.clear();
-  for (int k = 0; k < A; ++k)
-    for (int j = 0; j < B; ++j) {
-      const double a = -two_pi * (double)((long long)j * k % n) / (double)n;
-      tw.push_back(make_float2((float)std::cos(a), (float)std::sin(a)));
-    }
+  phased_twiddles(n, A, tw);
   pq.assign(n, make_float2(0.f, 0.f));
   for (int k = 0; k < n; ++k) {
     const int k1 = k % A, k2 = k / A, s = (p.tx == 8 && B % 2 == 0) ? k1 & 1 : 0;
@@ -393,12 +434,7 @@ inline RowPlan plan_rows(int n, long long rows, int sms, size_t budget, size_t f
 // Twiddles w_n^{j k1} at k1 B + j and the wave numbers of the natural order, for plan_rows' axes.
 inline void row_tables(int n, const RowPlan& p, std::vector<float2>& tw, std::vector<float2>& pq) {
   const double two_pi = 6.283185307179586476925287;
-  tw.clear();
-  for (int k = 0; k < p.A; ++k)
-    for (int j = 0; j < p.B; ++j) {
-      const double a = -two_pi * (double)((long long)j * k % n) / (double)n;
-      tw.push_back(make_float2((float)std::cos(a), (float)std::sin(a)));
-    }
+  phased_twiddles(n, p.A, tw);
   pq.assign(n, make_float2(0.f, 0.f));
   for (int k = 0; k < n; ++k) {
     const float q = (float)(two_pi * (double)((2 * k < n) ? k : k - n) / (double)n);
@@ -408,7 +444,7 @@ inline void row_tables(int n, const RowPlan& p, std::vector<float2>& tw, std::ve
 
 // Device tables of an axis for a given radix order (see fft_ip.cuh): the stage table
 // (2 int4 per stage), the twiddle table (complex64, w_n^{j k P_q} at tw_off_q + (k-1) m_q + j,
-// computed in FP64 and rounded), and the wave numbers (p, q) of each position (scaled by the
+// computed in FP64 and rounded as unit_pair says), and the wave numbers (p, q) of each position (scaled by the
 // pitch: p = 2 pi fftfreq(k, n), q = p but 0 at the Nyquist frequency of an even n).
 inline void axis_tables(int n, const std::vector<int>& order, std::vector<int4>& st, std::vector<float2>& tw,
                         std::vector<float2>& pq) {
@@ -433,7 +469,7 @@ inline void axis_tables(int n, const std::vector<int>& order, std::vector<int4>&
       for (int k = 1; k < R; ++k)
         for (int j = 0; j < m; ++j) {
           const double a = -two_pi * (double)((long long)j * k * P % n) / (double)n;
-          tw.push_back(make_float2((float)std::cos(a), (float)std::sin(a)));
+          tw.push_back(unit_twiddle(a));
         }
   }
   // position of frequency k: its mixed-radix digits d_q (d_0 least significant, base R_0)

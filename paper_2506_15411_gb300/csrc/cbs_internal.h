@@ -34,6 +34,7 @@ struct Member {
   SourceArgs src;
   float inv_eps;          // 1 / epsilon (scaled)
   float2 kt2;             // k0^2 + i epsilon (scaled)
+  int phase;              // of the twiddle tables at slot 0: iterations of its series before the block
   int seat;               // slice of the plan's arrays: E, W at + seat * 3 Nw; V at + seat * Nw
 };
 
@@ -89,6 +90,7 @@ struct IterArgs {
   const float2* twx;      // per-stage twiddle tables; each 128-byte aligned, padded to n entries
   const float2* twy;
   const float2* twz;
+  int twsx, twsy, twsz;   // from one phase's twiddles to the next (0: one table)
   int twbx, twby, twbz;   // bytes copied per table: n * 8 rounded up to a multiple of 16
   const float2* pqx;      // wave numbers (p, q) of each position of an axis' spectrum,
   const float2* pqy;      // padded with zeros to a multiple of 16 entries
@@ -100,7 +102,7 @@ struct IterArgs {
   int seats;              // requests the arrays hold
   int nmem;               // members of this launch (1 .. kMaxMembers)
   const Member* mem;      // their sources, splittings and seats (device memory)
-  float invN;             // 1 / N, folded into the k-space multiply
+  float invN, invN_rest;  // 1 / N, folded into the k-space multiply: invN (1 + invN_rest)
   double* partials;       // residual partial sums, [seat][kResidualSlots][grid_x]
   double* hist;           // hist[seat * hist_cap + slot] = sum |delta|^2 of this iteration
   int hist_cap;
@@ -138,6 +140,9 @@ CBS_HD size_t wrow(int y, int z, int nz, int yblk) {
   const int yb = y / yblk;
   return ((size_t)yb * nz + z) * yblk + (y - yb * yblk);
 }
+
+// The twiddle tables of this launch's iteration, for a member (axis_plan.h).
+CBS_HD int twiddle_phase(const IterArgs& a, const Member& m) { return (a.slot + m.phase) % kTwiddlePhases; }
 
 // Launchers (one per pass of an iteration); each returns the launch error.
 cudaError_t launch_xpass_fwd(const IterArgs& a, bool zero, cudaStream_t s);   // W = FFTx(V E + S); zero: E is 0

@@ -2,7 +2,7 @@
 //
 //   y pass:  W_c <- FFT_y(W_c) or IFFT_y(W_c), one (component, z) plane x TX columns per tile
 //   z pass:  W <- IFFT_z( G(p) FFT_z(W) ), the three components of one y row x TX columns,
-//            G(p) the dyadic Green's function of curl curl - kt2 (green() below), scaled by 1/N
+//            G(p) the dyadic Green's function of curl curl - kt2, scaled by 1/N (green.cuh)
 // (the k-space steps of the vector CBS of refs. [25], [26] of arXiv 2506.15411.)
 //
 // i = j + B r (j < B, r < A).  Step 1 of the forward transform: a thread takes one column's A
@@ -35,6 +35,7 @@
 #include "axis_plan.h"
 #include "cbs_internal.h"
 #include "fft_ip.cuh"
+#include "green.cuh"
 #include "tma.cuh"
 
 namespace cbs {
@@ -113,27 +114,6 @@ __device__ __forceinline__ void col_step2(float2* buf, int lt) {
   }
 }
 
-// The k-space multiply at wave vector p (q = p except 0 in a Nyquist component):
-//   X <- [X + q (q.X) f] d,  f = 1 / (|p|^2 - |q|^2 - kt2),  d = invN / (|p|^2 - kt2),
-// the inverse of |p|^2 I - q q^T - kt2 I (a Nyquist component is 0 in q, which keeps the discrete
-// curl curl real and symmetric).  f is the same at every z that is not Nyquist.
-__device__ __forceinline__ void green(float qx, float qy, float qz, float2 f, float p2, float2 kt2, float invN,
-                                      float2& X0, float2& X1, float2& X2) {
-  const float2 qd = cfma_r(qz, X2, cfma_r(qy, X1, make_float2(qx * X0.x, qx * X0.y)));
-  const float2 c = cmul(qd, f);
-  const float dr = p2 - kt2.x, di = -kt2.y;
-  const float sc = invN * __fdividef(1.0f, dr * dr + di * di);
-  const float2 d = make_float2(dr * sc, -di * sc);
-  X0 = cmul(cfma_r(qx, c, X0), d);
-  X1 = cmul(cfma_r(qy, c, X1), d);
-  X2 = cmul(cfma_r(qz, c, X2), d);
-}
-__device__ __forceinline__ float2 green_f(float nyq2, float2 kt2) {
-  const float cr = nyq2 - kt2.x, ci = -kt2.y;
-  const float s = __fdividef(1.0f, cr * cr + ci * ci);
-  return make_float2(cr * s, -ci * s);
-}
-
 template <int N, int KIND>
 __global__ void __launch_bounds__(col_plan(N, KIND == kZ ? 3 : 1).threads(), 1)
     k_col(const __grid_constant__ CUtensorMap tm, const IterArgs a) {
@@ -201,7 +181,8 @@ __global__ void __launch_bounds__(col_plan(N, KIND == kZ ? 3 : 1).threads(), 1)
     // the next tile into that set
     if (lane == 0) {
       mbar_arrive_expect_tx(tbar, twb + (KIND == kZ ? a.pqbz : 0));
-      bulk_load(tw, KIND == kZ ? a.twz : a.twy, twb, tbar);
+      const int phase = twiddle_phase(a, a.mem[mb.j]);
+      bulk_load(tw, KIND == kZ ? a.twz + phase * a.twsz : a.twy + phase * a.twsy, twb, tbar);
       if (KIND == kZ) bulk_load(pqz, a.pqz, a.pqbz, tbar);
     }
     const uint32_t bytes = (uint32_t)(tileN * sizeof(float2));
@@ -310,13 +291,11 @@ __global__ void __launch_bounds__(col_plan(N, KIND == kZ ? 3 : 1).threads(), 1)
       col_step1<A, B, TX, 3, GT, false>(cur, cs, tw, lt);
       gsync();
       constexpr bool SW = TX == 8 && B % 2 == 0;
-      const float nyq2 = (px.x * px.x - px.y * px.y) + (py.x * py.x - py.y * py.y);
-      const float pxy2 = px.x * px.x + py.x * py.x;
-      const float2 f = green_f(nyq2, kt2);
+      const GreenColumn col = green_column(px, py, kt2);
 #pragma unroll 1
       for (int m = lt; m < TX * A; m += GT) {
-        const int col = m % TX, k1 = m / TX;
-        float2* const q = cur + k1 * B * TX + col;
+        const int k1 = m / TX;
+        float2* const q = cur + k1 * B * TX + m % TX;
         const int sw = SW ? (k1 & 1) * TX : 0;
         float2* const qe = q + sw;
         float2* const qo = q - sw;
@@ -328,12 +307,8 @@ __global__ void __launch_bounds__(col_plan(N, KIND == kZ ? 3 : 1).threads(), 1)
           DFT<B, false>::run(v[c]);
         }
 #pragma unroll
-        for (int k2 = 0; k2 < B; ++k2) {
-          const float2 pz = pqz[k1 + A * k2];
-          float2 fz = f;
-          if (pz.x != pz.y) fz = green_f(nyq2 + pz.x * pz.x, kt2);   // z Nyquist (pz.y = 0)
-          green(px.y, py.y, pz.y, fz, fmaf(pz.x, pz.x, pxy2), kt2, a.invN, v[0][k2], v[1][k2], v[2][k2]);
-        }
+        for (int k2 = 0; k2 < B; ++k2)
+          green(col, pqz[k1 + A * k2], kt2, a.invN, a.invN_rest, v[0][k2], v[1][k2], v[2][k2]);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           DFT<B, true>::run(v[c]);

@@ -323,6 +323,7 @@ int enqueue_block(cbs_server_s* S, Batch* b) {
     s.blk = 0;
     if (s.phase != Phase::Forward && s.phase != Phase::Adjoint) continue;
     s.blk = std::min(p->d.check_every, p->d.max_iter - s.run.it);
+    s.mem.phase = s.run.it % kTwiddlePhases;
     L = std::max(L, s.blk);
   }
   if (L == 0) return CBS_OK;

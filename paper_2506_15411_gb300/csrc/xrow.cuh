@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
       const float2* const V = a.V + (size_t)mem.seat * a.Nw;
       if (lane == 0) {
         mbar_arrive_expect_tx(tbar, a.twbx);
-        bulk_load(tw, a.twx, a.twbx, tbar);
+        bulk_load(tw, a.twx + twiddle_phase(a, mem) * a.twsx, a.twbx, tbar);
       }
       wait_for_previous();
       int k = 0, n = 0;

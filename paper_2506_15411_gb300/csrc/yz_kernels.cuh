@@ -3,9 +3,8 @@
 //
 //   y pass:  W_c <- FFT_y(W_c) or IFFT_y(W_c), one (component, z) plane x TX columns per tile
 //   z pass:  W <- IFFT_z( G(p) FFT_z(W) ), the three components of one y row x TX columns,
-//            where G(p) = (I - p p^T / kt2) / (|p|^2 - kt2), kt2 = k0^2 + i epsilon, is the
-//            dyadic Green's function of curl curl - kt2 (the vector CBS of refs. [25], [26] of
-//            arXiv 2506.15411), scaled by 1/N for the inverse FFT (Nyquist treatment at green()).
+//            where G(p) is the dyadic Green's function of curl curl - kt2 (green.cuh), scaled by
+//            1/N for the inverse FFT
 //
 // Forward transforms are in-place decimation in frequency and leave each axis' spectrum in
 // digit-reversed order in W; inverse transforms are decimation in time and restore natural
@@ -25,32 +24,12 @@
 
 #include "cbs_internal.h"
 #include "fft_ip.cuh"
+#include "green.cuh"
 #include "tma.cuh"
 
 namespace cbs {
 
 namespace yzk {
-
-// k-space multiply at wave vector p (q = p except 0 in a Nyquist component):
-//   X <- [X + q (q.X) / (|p|^2 - |q|^2 - kt2)] * invN / (|p|^2 - kt2),
-// the inverse of |p|^2 I - q q^T - kt2 I.  A Nyquist component (even axis length, wave number
-// pi/pitch whose sign is undefined) is 0 in q, which keeps the discrete curl curl real and
-// symmetric.  Away from Nyquist q = p and this is (I - p p^T / kt2) / (|p|^2 - kt2).
-__device__ __forceinline__ void green(float px, float py, float pz, float qx, float qy, float qz, float2 kt2,
-                                      float invN, float2& X0, float2& X1, float2& X2) {
-  const float p2 = px * px + py * py + pz * pz;
-  const float nyq2 = (px * px - qx * qx) + (py * py - qy * qy) + (pz * pz - qz * qz);
-  const float cr = nyq2 - kt2.x, ci = -kt2.y;
-  const float cs = __fdividef(1.0f, cr * cr + ci * ci);
-  const float2 qd = make_float2(qx * X0.x + qy * X1.x + qz * X2.x, qx * X0.y + qy * X1.y + qz * X2.y);
-  const float2 c = cmul(qd, make_float2(cr * cs, -ci * cs));
-  const float dr = p2 - kt2.x, di = -kt2.y;
-  const float sc = invN * __fdividef(1.0f, dr * dr + di * di);
-  const float2 inv = make_float2(dr * sc, -di * sc);   // invN / (dr + i di)
-  X0 = cmul(make_float2(X0.x + qx * c.x, X0.y + qx * c.y), inv);
-  X1 = cmul(make_float2(X1.x + qy * c.x, X1.y + qy * c.y), inv);
-  X2 = cmul(make_float2(X2.x + qz * c.x, X2.y + qz * c.y), inv);
-}
 
 #ifndef CBS_Y_THREADS
 #define CBS_Y_THREADS 512
@@ -262,13 +241,12 @@ __global__ void __launch_bounds__(kZThreads, kZOcc) k_zpass_green(const __grid_c
     // the fused stage gives thread lt the items lt, lt + GT, ...: all in column lt mod TX, as
     // GT is a multiple of TX; so its x wave number is read once per tile (the table is padded
     // past nx)
-    const float2 px = __ldg(&a.pqx[x0 + lt % TX]);
+    const GreenColumn col = green_column(__ldg(&a.pqx[x0 + lt % TX]), pqy, kt2);
     col_stages<false, TX, 3, MAXR, true>(cur, cs, a.az, 0, ns - 1, tw, lt, GT, prefetch, gsync);
     radix_dispatch<MAXR>(sl.R, [&](auto Ri) {
       constexpr int R = decltype(Ri)::value;
       ipz_fused<R, TX>(cur, cs, sl, lt, GT, [&](int, int pos, float2& X0, float2& X1, float2& X2) {
-        const float2 pz = pqz[pos];
-        green(px.x, pqy.x, pz.x, px.y, pqy.y, pz.y, kt2, a.invN, X0, X1, X2);
+        green(col, pqz[pos], kt2, a.invN, a.invN_rest, X0, X1, X2);
       });
     });
     gsync();
