@@ -372,6 +372,11 @@ int cbs_server_sharing(cbs_server_t server, long long* launches, long long* requ
  * or CBS_ERR_CUDA with a message. */
 int cbs_selftest_wait_timeout(int* device_status);
 
+/* Let the tile waits of a plan's kernels give up after `polls` polls (0: at once, as if the copy had
+ * not come; negative: back to the usual limit).  For tests of the failure path: a solve then ends with
+ * CBS_ERR_CUDA, the last iterate is of no use, and the plan stays usable. */
+int cbs_selftest_wait_limit(cbs_plan_t plan, long long polls);
+
 /* Free the plan and its device memory (NULL is a no-op). */
 void cbs_destroy(cbs_plan_t plan);
 

@@ -871,6 +871,7 @@ int plan_create(cbs_plan_s** out, const cbs_plan_desc* desc, int seats) {
   a.nmem = 1;
   a.mem = p->mem_dev;
   a.err = p->err_dev;
+  a.wait_limit = kWaitLimit;
   a.partials = p->partials;
   a.hist = p->hist;
   a.hist_cap = d.check_every;
@@ -1082,6 +1083,14 @@ int cbs_selftest_wait_timeout(int* device_status) {
   if (e != cudaSuccess) return fail(CBS_ERR_CUDA, "self-test: %s", cudaGetErrorString(e));
   if (*device_status != kErrTmaTimeout)
     return fail(CBS_ERR_CUDA, "self-test: the bounded wait did not report its timeout (status %d)", *device_status);
+  return CBS_OK;
+}
+
+int cbs_selftest_wait_limit(cbs_plan_t p, long long polls) {
+  g_err.clear();
+  if (!p) return fail(CBS_ERR_ARG, "NULL argument");
+  drop_graphs(p);   // (the limit is among their kernels' arguments)
+  p->base.wait_limit = polls < 0 ? kWaitLimit : polls;
   return CBS_OK;
 }
 

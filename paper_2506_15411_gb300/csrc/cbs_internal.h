@@ -108,6 +108,7 @@ struct IterArgs {
   int hist_cap;
   int slot;
   int* err;               // device error flag (a tensor-copy wait that timed out)
+  long long wait_limit;   // polls after which a wait on a tile gives up
   // launch shapes
   XRowShape xr;
   ColShape yc, zc;

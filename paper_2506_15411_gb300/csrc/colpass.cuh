@@ -134,6 +134,7 @@ __global__ void __launch_bounds__(col_plan(N, KIND == kZ ? 3 : 1).threads(), 1)
   uint64_t* const tbar = done + S;
   volatile int* const flags = reinterpret_cast<volatile int*>(tbar + 1);   // a wait gave up
   volatile int* const issued = flags + 1;                                    // tiles issued so far
+  int* const bad = reinterpret_cast<int*>(tbar + 1) + 2;                     // tiles misaligned
   const int nxt = (a.nx + TX - 1) / TX;
   const int ntiles = KIND == kZ ? nxt * a.ny : nxt * a.nz * 3;
   const int G = KIND == kZ ? a.grid_z : a.grid_y;
@@ -142,8 +143,9 @@ __global__ void __launch_bounds__(col_plan(N, KIND == kZ ? 3 : 1).threads(), 1)
   if (mb.b >= ntiles) return;
   const int tid = threadIdx.x, lane = tid & 31;
   if (tid == 0) {
-    *flags = (smem_u32(buf0) & 127u) ? 1 : 0;
-    if (*flags) atomicExch(a.err, kErrMisaligned);
+    *bad = (smem_u32(buf0) & 127u) ? 1 : 0;
+    if (*bad) atomicExch(a.err, kErrMisaligned);
+    *flags = 0;
     *issued = 0;
     for (int i = 0; i < S; ++i) {
       mbar_init(full + i, 1);
@@ -153,7 +155,7 @@ __global__ void __launch_bounds__(col_plan(N, KIND == kZ ? 3 : 1).threads(), 1)
     fence_mbar_init();
   }
   __syncthreads();
-  if (*flags) return;
+  if (*bad) return;
   launch_dependents();
 
   const int n = (ntiles - mb.b + G - 1) / G;   // tiles of the block: mb.b, mb.b + G, ...
@@ -166,13 +168,18 @@ __global__ void __launch_bounds__(col_plan(N, KIND == kZ ? 3 : 1).threads(), 1)
     c = r / a.nz;
   };
 
-  // A wait that gives up records the error and raises the block's flag; later waits of the block
-  // then return at once and every thread runs on through the same barriers (on stale data; the
-  // host drops the result).
-  auto wait = [&](uint64_t* bar, uint32_t parity) {
-    if (*flags || mbar_wait(bar, parity)) return;
+  // A wait that gives up records the error and raises the block's flag.  The groups' later waits of
+  // the block then return at once and every thread runs on through the same barriers (on stale
+  // data; the host drops the result).  The copying warp stops: a set that was passed on unwaited for
+  // may still have its copy under way, and its mbarrier cannot be armed for another.  Then it waits
+  // until all it has loaded has landed, as the block may not end before; else every tile has been
+  // waited for by the time the last one is done.
+  auto give_up = [&] {
     *flags = 1;
     atomicExch(a.err, kErrTmaTimeout);
+  };
+  auto wait = [&](uint64_t* bar, uint32_t parity) {
+    if (!*flags && !mbar_wait(bar, parity, a.wait_limit)) give_up();
   };
 
   if (tid >= NG * GT) {
@@ -207,20 +214,29 @@ __global__ void __launch_bounds__(col_plan(N, KIND == kZ ? 3 : 1).threads(), 1)
           tma_load_5d(dst + b * box * TX, &tm, xt * TX, 0, z, b, c0 + c, full + k);
       }
     };
+    // (whoever passed a set on without its wait has raised the flag before, and then this gives up)
+    auto tile_done = [&](int k, uint32_t ph) { return warp_wait<true>(done + k, ph, flags, a.err, a.wait_limit); };
+    bool ok = true;
+    auto landed = [&] {
+      const int sent = *issued;   // (this warp's own count)
+      settle(full, S, max(0, sent - S), sent - 1);
+      mbar_wait(tbar, 0);
+    };
     wait_for_previous();
     for (int i = 0; i < min(S, n); ++i) load(mb.b + i * G, i);
     if constexpr (!COPY) {
       int k = 0;
       uint32_t ph = 0;
-      for (int i = S; i < n; ++i) {
-        wait(done + k, ph);
-        __syncwarp();
-        load(mb.b + i * G, k);
+      for (int i = 0; i < n; ++i) {   // tile i's set takes tile i + S
+        ok = tile_done(k, ph);
+        if (!ok) break;
+        if (i + S < n) load(mb.b + (i + S) * G, k);
         if (++k == S) {
           k = 0;
           ph ^= 1u;
         }
       }
+      if (!ok) landed();
       return;
     }
     const int lag = S >= NG + 2 ? 1 : 0;
@@ -228,8 +244,8 @@ __global__ void __launch_bounds__(col_plan(N, KIND == kZ ? 3 : 1).threads(), 1)
     uint32_t ph = 0;
     for (int i = 0; i < n; ++i) {
       const int t = mb.b + i * G;
-      wait(done + k, ph);
-      __syncwarp();
+      ok = tile_done(k, ph);
+      if (!ok) break;
       const float2* const src = buf0 + k * tileN;
       if constexpr (KIND == kZ) {
         const int xt = t % nxt, y = t / nxt, yb = y / a.yblk, yi = y - yb * a.yblk;
@@ -256,6 +272,7 @@ __global__ void __launch_bounds__(col_plan(N, KIND == kZ ? 3 : 1).threads(), 1)
         ph ^= 1u;
       }
     }
+    if (!ok) landed();
     bulk_wait_all();
     return;
   }
@@ -270,8 +287,8 @@ __global__ void __launch_bounds__(col_plan(N, KIND == kZ ? 3 : 1).threads(), 1)
     const int t = mb.b + i * G, u = i / S, k = i - u * S;
     // the set's use u is armed once the tile counts as issued: before that its mbarrier may still
     // be two phases back, where the parity alone would let the wait through
-    for (long long left = kWaitLimit; *issued <= i && !*flags;) {
-      if (--left == 0) *flags = 1;
+    for (long long left = a.wait_limit; *issued <= i && !*flags;) {
+      if (--left <= 0) give_up();
       __nanosleep(32);
     }
     wait(full + k, (uint32_t)(u & 1));

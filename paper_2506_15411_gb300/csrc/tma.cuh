@@ -52,6 +52,28 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
   return false;
 }
 
+// The same for a warp that works as one (all 32 lanes call it): the lanes' verdicts are joined, so
+// that none goes on where another gives up.  A wait that is not over at once gives up where another
+// warp has set *failed (STRICT: also one that is), and sets it (and *err) when it gives up.
+template <bool STRICT = false>
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* failed, int* err,
+                                          long long limit) {
+  bool ok = limit > 0 && mbar_try_wait(bar, parity);
+  for (long long i = 1; i < limit && !ok && !*failed; ++i) ok = mbar_try_wait(bar, parity);
+  ok = __all_sync(0xffffffffu, STRICT ? ok && !*failed : ok);
+  if (!ok && (threadIdx.x & 31) == 0) {
+    *failed = 1;
+    atomicExch(err, kErrTmaTimeout);
+  }
+  return ok;
+}
+
+// The copies of tiles first, first + step, ... last of a ring of n sets (tile i in set i mod n) have
+// landed, or the waits' limit is over: what a thread that issued them does before it may leave.
+__device__ __forceinline__ void settle(uint64_t* full, int n, int first, int last, int step = 1) {
+  for (int i = first; i <= last; i += step) mbar_wait(full + i % n, (uint32_t)((i / n) & 1));
+}
+
 // 4D tiled tensor load global -> shared (completion counted on `bar` in bytes).
 __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* tm, int c0, int c1, int c2, int c3,
                                             uint64_t* bar) {
@@ -141,8 +163,8 @@ __device__ __forceinline__ bool block_setup_n(const void* tile, uint64_t* bars, 
 
 // Bounded wait for phase `parity` of a tile's copies, shared by the block: every thread
 // polls; a timeout anywhere aborts the whole block (uniformly) and records an error.
-__device__ __forceinline__ bool block_wait(uint64_t* bar, int* fail, int* err, uint32_t parity = 0) {
-  if (!mbar_wait(bar, parity)) *fail = 1;
+__device__ __forceinline__ bool block_wait(uint64_t* bar, int* fail, int* err, uint32_t parity, long long limit) {
+  if (!mbar_wait(bar, parity, limit)) *fail = 1;
   __syncthreads();
   if (*fail) {
     if (threadIdx.x == 0) atomicExch(err, kErrTmaTimeout);

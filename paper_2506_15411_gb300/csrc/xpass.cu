@@ -154,7 +154,13 @@ __global__ void __launch_bounds__(kThreads, kXOcc) k_xpass_fwd(const IterArgs a)
   int k = 0;
   for (int i = 0, tile = mb.b; tile < ntiles; ++i, tile += G, k = (k + 1 == nset) ? 0 : k + 1) {
     const int r0 = tile * rpb, nr = min(rpb, rows - r0);
-    if (!block_wait(&t.full[k], t.fail, a.err, (uint32_t)((i / nset) & 1))) return;
+    if (!block_wait(&t.full[k], t.fail, a.err, (uint32_t)((i / nset) & 1), a.wait_limit)) {
+      if (tid == 0) {   // (the block may not end before its copies have landed)
+        settle(t.full, nset, i, min(i + nset - 2, (ntiles - 1 - mb.b) / G));
+        bulk_wait_all();
+      }
+      return;
+    }
     float2* e = t.set0 + k * t.set;
     const float2* v = e + 3 * span;
     auto prefetch = [&] {
@@ -246,7 +252,7 @@ __global__ void __launch_bounds__(kThreads, kXOcc) k_xpass_inv_fwd(const IterArg
       else group_sync_x(1 + g, GT);
     };
     auto gwait = [&](uint64_t* bar, uint32_t parity) {
-      if (!mbar_wait(bar, parity)) t.fail[g] = 1;
+      if (!mbar_wait(bar, parity, a.wait_limit)) t.fail[g] = 1;
       gsync();
       if (t.fail[g]) {
         if (lt == 0) atomicExch(a.err, kErrTmaTimeout);
@@ -258,11 +264,24 @@ __global__ void __launch_bounds__(kThreads, kXOcc) k_xpass_inv_fwd(const IterArg
     const RowDecode rowdec = row_decode(a);
     const int ns = a.ax.ns;
     const IPStage s0 = ip_decode_stage(a.ax, 0);
+    // what a group's leader has issued from its tile i on has landed (as in the z pass)
+    auto leave = [&](int i) {
+      if (lt != 0) return;
+      const int last = (ntiles - 1 - mb.b) / G;
+      for (int j = i - NG + D; j >= max(D, i - NG + 1); j -= NG)
+        if (j <= last) settle(t.full, nset, j, j);
+      if (tid == 0) {
+        mbar_wait(t.tbar, 0);
+        settle(t.full, nset, max(0, i - NG + 1), min(D - 1, last));
+      }
+    };
     bool ok = gwait(t.tbar, 0);
+    if (!ok) leave(g);
     for (int i = g, tile = mb.b + g * G; ok && tile < ntiles; i += NG, tile += NG * G) {
       const int k = i % nset;
       const int r0 = tile * rpb, nr = min(rpb, rows - r0);
       if (!gwait(&t.full[k], (uint32_t)((i / nset) & 1))) {
+        leave(i);
         ok = false;
         break;
       }

@@ -18,7 +18,9 @@
 //
 // A block is persistent: T teams of three warps, one warp per field component, and a producer
 // warp that keeps S tiles of rpb rows (W, E of three components, V) in flight or in hand.  A
-// team's warps meet only at the mbarriers of their tile; each warp stores its own component.
+// team's warps meet only at the mbarriers of their tile; each warp stores its own component.  A
+// wait that gives up does so for its whole warp and raises the block's flag, at which the others give
+// up too; all meet at the block's end, the producer once its copies have landed.
 //
 // Bound by memory: 104 bytes a voxel.  The staged pass (xpass.cu) spent its time at barriers and
 // on shared memory, which its three or four stages cross 17 times per value, and on their bank
@@ -107,8 +109,9 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
   uint64_t* const full = reinterpret_cast<uint64_t*>(tw + a.twbx / sizeof(float2));   // [S]
   uint64_t* const empty = full + S;                                                   // [S]
   uint64_t* const tbar = empty + S;
-  int* const flags = reinterpret_cast<int*>(tbar + 1);   // alignment failure
-  volatile int* const issued = flags + 1;                // tiles of the block issued so far
+  volatile int* const failed = reinterpret_cast<volatile int*>(tbar + 1);   // a wait gave up
+  volatile int* const issued = failed + 1;                                  // tiles of the block issued so far
+  int* const bad = reinterpret_cast<int*>(tbar + 1) + 2;                    // tiles misaligned
 
   const MemberBlock mb = member_block(blockIdx.x, G);
   const Member& mem = a.mem[mb.j];
@@ -117,8 +120,9 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
   float acc = 0.f;
   if (mb.b < ntiles) {
     if (tid == 0) {
-      flags[0] = (smem_u32(set0) & 127u) ? 1 : 0;
-      if (flags[0]) atomicExch(a.err, kErrMisaligned);
+      *bad = (smem_u32(set0) & 127u) ? 1 : 0;
+      if (*bad) atomicExch(a.err, kErrMisaligned);
+      *failed = 0;
       for (int i = 0; i < S; ++i) {
         mbar_init(full + i, 1);
         mbar_init(empty + i, 3);
@@ -128,7 +132,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
       fence_mbar_init();
     }
     __syncthreads();
-    if (flags[0]) return;   // (uniform)
+    if (*bad) return;
     launch_dependents();
     const uint32_t rb = (uint32_t)(((a.nx + 1) & ~1) * sizeof(float2));   // bytes of a row copy
     if (warp == 3 * T) {
@@ -144,10 +148,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
       int k = 0, n = 0;
       uint32_t ph = 1;   // a fresh mbarrier passes a wait for the phase before its first
       for (int tile = mb.b; tile < ntiles; tile += G) {
-        if (!mbar_wait(empty + k, ph)) {
-          if (lane == 0) atomicExch(a.err, kErrTmaTimeout);
-          break;
-        }
+        if (!warp_wait(empty + k, ph, failed, a.err, a.wait_limit)) break;
         const int r0 = tile * rpb, nr = min(rpb, rows - r0);
         if (lane == 0) {
           mbar_arrive_expect_tx(full + k, (mode == 0 ? 7 : (mode == 1 ? 4 : 0)) * nr * rb);
@@ -173,6 +174,11 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
           ph ^= 1u;
         }
       }
+      // no copy may be under way when the sums below go over the tiles, or the block ends: a team
+      // that gave up has not waited for its own
+      settle(full, S, max(0, n - S), n - 1);
+      mbar_wait(tbar, 0);
+      __syncwarp();
     } else {
       const int team = warp / 3, c = warp - 3 * team;
       const int skind = mem.src.kind, splane = skind == 1 ? mem.src.pz : mem.src.zp;
@@ -184,18 +190,25 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
       float2* const Wg = a.W + so + c * a.Nw;
       constexpr int per = 32 / B;   // rows of a round of step 1
       const int lr = lane / B, j = lane - lr * B;
-      bool ok = mbar_wait(tbar, 0);
+      bool ok = warp_wait(tbar, 0, failed, a.err, a.wait_limit);
 #pragma unroll 1
       for (int i = team, tile = mb.b + team * G; ok && tile < ntiles; i += T, tile += T * G) {
         const int u = i / S, k = i - u * S;
         // the set's use u is armed once the tile counts as issued: before that its mbarrier may
         // still be two phases back, where the parity alone would let the wait through
-        long long left = kWaitLimit;
-        while (*issued <= i && --left > 0) __nanosleep(32);
-        if (left <= 0 || !mbar_wait(full + k, (uint32_t)(u & 1))) {
-          ok = false;
+        bool on = *issued > i;
+        for (long long left = a.wait_limit; !on && !*failed && left > 0; --left) {
+          __nanosleep(32);
+          on = *issued > i;
+        }
+        if (!__all_sync(0xffffffffu, on)) {
+          if (lane == 0) {
+            *failed = 1;
+            atomicExch(a.err, kErrTmaTimeout);
+          }
           break;
         }
+        if (!warp_wait(full + k, (uint32_t)(u & 1), failed, a.err, a.wait_limit)) break;
         const int r0 = tile * rpb, nr = min(rpb, rows - r0);
         float2* const w = set0 + k * set + c * rpb * ldw;
         float2* const e = set0 + k * set + 3 * rpb * ldw + c * rpb * lde;
@@ -291,12 +304,11 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
         }
         __syncwarp();
       }
-      if (!ok && lane == 0) atomicExch(a.err, kErrTmaTimeout);
     }
   }
   if (mode == 0) {
-    // the block's residual: the threads' sums through shared memory (every tile has been read out
-    // of it by now), one warp adds them in FP64 in a fixed order
+    // the block's residual: the threads' sums through shared memory (every copy into it has landed
+    // and every tile been read out of it by now), one warp adds them in FP64 in a fixed order
     float* const sums = reinterpret_cast<float*>(smem_raw);
     __syncthreads();
     sums[tid] = acc;

@@ -127,7 +127,13 @@ __global__ void __launch_bounds__(y_threads<OCC>(), OCC) k_ypass(const __grid_co
   int b = 0;
   for (int i = 0, t = mb.b; t < ntiles; ++i, t += G, b = (b + 1 == nbuf) ? 0 : b + 1) {
     float2* cur = buf0 + b * tileN;
-    if (!block_wait(&full[b], fail, a.err, (uint32_t)((i / nbuf) & 1))) return;
+    if (!block_wait(&full[b], fail, a.err, (uint32_t)((i / nbuf) & 1), a.wait_limit)) {
+      if (tid == 0) {   // (the block may not end before its copies have landed)
+        settle(full, nbuf, i, min(i + nbuf - 2, (ntiles - 1 - mb.b) / G));
+        bulk_wait_all();
+      }
+      return;
+    }
     auto prefetch = [&] {
       const int tn = t + (nbuf - 1) * G;
       if (tid == 0 && tn < ntiles) {
@@ -213,7 +219,7 @@ __global__ void __launch_bounds__(kZThreads, kZOcc) k_zpass_green(const __grid_c
   };
   // bounded wait of the group on an mbarrier phase; a timeout aborts the group uniformly
   auto gwait = [&](uint64_t* bar, uint32_t parity) {
-    if (!mbar_wait(bar, parity)) fail[g] = 1;
+    if (!mbar_wait(bar, parity, a.wait_limit)) fail[g] = 1;
     gsync();
     if (fail[g]) {
       if (lt == 0) atomicExch(a.err, kErrTmaTimeout);
@@ -221,13 +227,32 @@ __global__ void __launch_bounds__(kZThreads, kZOcc) k_zpass_green(const __grid_c
     }
     return true;
   };
-  if (!gwait(tbar, 0)) return;
+  // what a group's leader has issued from its tile i on (for the tiles i - NG + D, i - 2 NG + D, ...; the
+  // block's first thread also the first D tiles and the tables) has landed
+  auto leave = [&](int i) {
+    if (lt != 0) return;
+    const int last = (ntiles - 1 - mb.b) / G;
+    for (int j = i - NG + D; j >= max(D, i - NG + 1); j -= NG)
+      if (j <= last) settle(full, nbuf, j, j);
+    if (tid == 0) {
+      mbar_wait(tbar, 0);
+      settle(full, nbuf, max(0, i - NG + 1), min(D - 1, last));
+    }
+    bulk_wait_all();
+  };
+  if (!gwait(tbar, 0)) {
+    leave(g);
+    return;
+  }
   const int ns = a.az.ns;
   const IPStage sl = ip_decode_stage(a.az, ns - 1);
   for (int i = g, t = mb.b + g * G; t < ntiles; i += NG, t += NG * G) {
     const int b = i % nbuf;
     float2* cur = buf0 + b * tileN;
-    if (!gwait(&full[b], (uint32_t)((i / nbuf) & 1))) return;
+    if (!gwait(&full[b], (uint32_t)((i / nbuf) & 1))) {
+      leave(i);
+      return;
+    }
     auto prefetch = [&] {
       const int tn = t + D * G;
       if (lt == 0 && tn < ntiles) {
