@@ -122,7 +122,7 @@ __global__ void k_k2_maxdev(const float* __restrict__ eps, int nx, int ny, int n
   const float kv2f = (float)kv2, k0f = (float)k0sq;
   const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
   double m = 0.0;
-  float mf = 0.f;   // at most m
+  float mf = -1.f;   // at most m; -1 while m is so small that a bound's squares may underflow
   float eh = 0.f;   // permittivity and row part of the lane's last voxel between the layers
   double imh = -1.0;
   for (int row = blockIdx.x * warps + (threadIdx.x >> 5); row < ny * nz; row += gridDim.x * warps) {
@@ -146,7 +146,7 @@ __global__ void k_k2_maxdev(const float* __restrict__ eps, int nx, int ny, int n
         if (__any_sync(0xffffffffu, !skip)) {
           // squared: one square root per block, not per voxel
           m = fmax(m, dev2(e[k], inner ? 0.0 : sx[x], syr, szr, corner_max, kv2, k0sq));
-          mf = __double2float_rd(m);
+          mf = m < 1e-30 ? -1.f : __double2float_rd(m);
           if (inner) {
             eh = e[k];
             imh = im0;
