@@ -146,7 +146,8 @@ __global__ void k_k2_maxdev(const float* __restrict__ eps, int nx, int ny, int n
         if (__any_sync(0xffffffffu, !skip)) {
           // squared: one square root per block, not per voxel
           m = fmax(m, dev2(e[k], inner ? 0.0 : sx[x], syr, szr, corner_max, kv2, k0sq));
-          mf = m < 1e-30 ? -1.f : __double2float_rd(m);
+          mf = __double2float_rd(m);
+          if (mf < 1e-30f) mf = -1.f;
           if (inner) {
             eh = e[k];
             imh = im0;
