@@ -1090,7 +1090,7 @@ int cbs_selftest_wait_limit(cbs_plan_t p, long long polls) {
   g_err.clear();
   if (!p) return fail(CBS_ERR_ARG, "NULL argument");
   drop_graphs(p);   // (the limit is among their kernels' arguments)
-  p->base.wait_limit = polls < 0 ? kWaitLimit : polls;
+  p->base.wait_limit = polls < 0 ? kWaitLimit : (unsigned)std::min<long long>(polls, kWaitLimit);
   return CBS_OK;
 }
 

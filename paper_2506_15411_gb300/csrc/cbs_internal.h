@@ -42,7 +42,10 @@ struct Member {
 // processors as the blocks of the one before leave them.  That saves 4 us an iteration where it
 // lasts tens (64^3 32.2 -> 28.6 us, 128^3 96.0 -> 91.5, 192 x 192 x 128 193 -> 191), but the blocks
 // then land on processors in any order, and neighbouring tiles, which share memory lines, on
-// both dies: 175 x 175 x 198 284 -> 290 us, 640 x 640 x 336 5.7 -> 6.6 ms.
+// both dies: 175 x 175 x 198 284 -> 290 us, 640 x 640 x 336 5.7 -> 6.6 ms.  The members of a launch do
+// not count: their tiles share no lines, and each brings a wave of blocks of its own (eight of
+// 192 x 192 x 128, 32 iterations and half as many adjoints: 77.9 ms, plain launches 78.7; eight of 128^3
+// 40.0, 40.7; eight of 112 x 108 x 96 26.8, 27.3; four of 160 x 150 x 140 30.1, 30.8; two 14.3, 14.3).
 constexpr size_t kOverlapVoxels = 5000000;
 
 // Launch a kernel that calls wait_for_previous() before it touches what the kernel before it in
@@ -108,7 +111,7 @@ struct IterArgs {
   int hist_cap;
   int slot;
   int* err;               // device error flag (a tensor-copy wait that timed out)
-  long long wait_limit;   // polls after which a wait on a tile gives up
+  unsigned wait_limit;    // polls after which a wait on a tile gives up
   // launch shapes
   XRowShape xr;
   ColShape yc, zc;

@@ -21,12 +21,12 @@
 // stores (128^3: 0.0225 -> 0.0184 ms; the other way 256 x 256 x 192: 0.104 -> 0.099).
 //
 // Bounds and figures (ms, one GB300; staged passes of yz_kernels.cuh -> these).  y, 48 bytes a
-// voxel, is bound by memory on large grids: 640 x 640 x 336 1.155 -> 1.10 (5.98 TB/s, 0.88 of a
-// copy), 384 x 384 x 256 0.290 -> 0.290, 175 x 175 x 198 0.070 -> 0.050, 104 x 104 x 120 (a factor
-// 13) 0.039 -> 0.0165, 128^3 0.030 -> 0.019.  z, also 48 bytes, by instruction issue and shared
-// memory, about half of each busy: 640 x 640 x 336 1.88 -> 1.36 (0.71 of a copy), 384 x 384 x 256
-// 0.616 -> 0.338 (0.79), 275 x 275 x 315 0.371 -> 0.302, 256 x 256 x 192 0.165 -> 0.111 (0.80),
-// 128^3 0.045 -> 0.025.  The staged passes took three to four stages each way, a barrier and a
+// voxel, is bound by memory on large grids: 640 x 640 x 336 1.155 -> 1.09 (6.06 TB/s, 0.89 of a
+// copy), 384 x 384 x 256 0.290 -> 0.294, 175 x 175 x 198 0.070 -> 0.051, 104 x 104 x 120 (a factor
+// 13) 0.039 -> 0.0167, 128^3 0.030 -> 0.0205.  z, also 48 bytes, by instruction issue and shared
+// memory, about half of each busy: 640 x 640 x 336 1.88 -> 1.35 (0.72 of a copy), 384 x 384 x 256
+// 0.616 -> 0.342 (0.78), 275 x 275 x 315 0.371 -> 0.293, 256 x 256 x 192 0.165 -> 0.112 (0.80),
+// 128^3 0.045 -> 0.0264.  The staged passes took three to four stages each way, a barrier and a
 // trip through shared memory each, with offsets computed at run time.
 #pragma once
 #include <algorithm>
@@ -173,10 +173,16 @@ __global__ void __launch_bounds__(col_plan(N, KIND == kZ ? 3 : 1).threads(), 1)
   // data; the host drops the result).  The copying warp stops: a set that was passed on unwaited for
   // may still have its copy under way, and its mbarrier cannot be armed for another.  Then it waits
   // until all it has loaded has landed, as the block may not end before; else every tile has been
-  // waited for by the time the last one is done.
+  // waited for by the time the last one is done.  Where it does not see the last ones (small y tiles),
+  // the groups do so too: either the flag was up by its last load, or that load counted before.
   auto give_up = [&] {
     *flags = 1;
     atomicExch(a.err, kErrTmaTimeout);
+  };
+  auto landed = [&] {
+    const int sent = *issued;
+    settle(full, S, max(0, sent - S), sent - 1);
+    mbar_wait(tbar, 0);
   };
   auto wait = [&](uint64_t* bar, uint32_t parity) {
     if (!*flags && !mbar_wait(bar, parity, a.wait_limit)) give_up();
@@ -217,26 +223,21 @@ __global__ void __launch_bounds__(col_plan(N, KIND == kZ ? 3 : 1).threads(), 1)
     // (whoever passed a set on without its wait has raised the flag before, and then this gives up)
     auto tile_done = [&](int k, uint32_t ph) { return warp_wait<true>(done + k, ph, flags, a.err, a.wait_limit); };
     bool ok = true;
-    auto landed = [&] {
-      const int sent = *issued;   // (this warp's own count)
-      settle(full, S, max(0, sent - S), sent - 1);
-      mbar_wait(tbar, 0);
-    };
     wait_for_previous();
     for (int i = 0; i < min(S, n); ++i) load(mb.b + i * G, i);
     if constexpr (!COPY) {
       int k = 0;
       uint32_t ph = 0;
-      for (int i = 0; i < n; ++i) {   // tile i's set takes tile i + S
+      for (int i = S; i < n; ++i) {
         ok = tile_done(k, ph);
         if (!ok) break;
-        if (i + S < n) load(mb.b + (i + S) * G, k);
+        load(mb.b + i * G, k);
         if (++k == S) {
           k = 0;
           ph ^= 1u;
         }
       }
-      if (!ok) landed();
+      if (!ok || *flags) landed();
       return;
     }
     const int lag = S >= NG + 2 ? 1 : 0;
@@ -287,10 +288,8 @@ __global__ void __launch_bounds__(col_plan(N, KIND == kZ ? 3 : 1).threads(), 1)
     const int t = mb.b + i * G, u = i / S, k = i - u * S;
     // the set's use u is armed once the tile counts as issued: before that its mbarrier may still
     // be two phases back, where the parity alone would let the wait through
-    for (long long left = a.wait_limit; *issued <= i && !*flags;) {
-      if (--left <= 0) give_up();
-      __nanosleep(32);
-    }
+    for (unsigned left = a.wait_limit; *issued <= i && !*flags; __nanosleep(32))
+      if (left-- <= 1) give_up();
     wait(full + k, (uint32_t)(u & 1));
     float2* const cur = buf0 + k * tileN;
     if constexpr (KIND == kYFwd) {
@@ -356,7 +355,10 @@ __global__ void __launch_bounds__(col_plan(N, KIND == kZ ? 3 : 1).threads(), 1)
       }
     }
   }
-  if constexpr (!COPY) bulk_wait_all();
+  if constexpr (!COPY) {
+    if (*flags) landed();
+    bulk_wait_all();
+  }
 }
 
 }  // namespace colk

@@ -11,7 +11,7 @@
 
 namespace cbs {
 
-constexpr long long kWaitLimit = 1LL << 24;   // polls of try_wait (each may suspend briefly)
+constexpr unsigned kWaitLimit = 1u << 24;   // polls of try_wait (each may suspend briefly)
 constexpr int kErrTmaTimeout = 1;
 constexpr int kErrMisaligned = 2;
 
@@ -46,8 +46,8 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 }
 
 // Bounded wait for phase `parity` of an mbarrier; false on timeout.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long long limit = kWaitLimit) {
-  for (long long i = 0; i < limit; ++i)
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, unsigned limit = kWaitLimit) {
+  for (unsigned i = 0; i < limit; ++i)
     if (mbar_try_wait(bar, parity)) return true;
   return false;
 }
@@ -57,9 +57,9 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
 // warp has set *failed (STRICT: also one that is), and sets it (and *err) when it gives up.
 template <bool STRICT = false>
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* failed, int* err,
-                                          long long limit) {
+                                          unsigned limit) {
   bool ok = limit > 0 && mbar_try_wait(bar, parity);
-  for (long long i = 1; i < limit && !ok && !*failed; ++i) ok = mbar_try_wait(bar, parity);
+  for (unsigned i = 1; i < limit && !ok && !*failed; ++i) ok = mbar_try_wait(bar, parity);
   ok = __all_sync(0xffffffffu, STRICT ? ok && !*failed : ok);
   if (!ok && (threadIdx.x & 31) == 0) {
     *failed = 1;
@@ -74,27 +74,9 @@ __device__ __forceinline__ void settle(uint64_t* full, int n, int first, int las
   for (int i = first; i <= last; i += step) mbar_wait(full + i % n, (uint32_t)((i / n) & 1));
 }
 
-// 4D tiled tensor load global -> shared (completion counted on `bar` in bytes).
-__device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* tm, int c0, int c1, int c2, int c3,
-                                            uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(tm)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(smem_u32(bar))
-      : "memory");
-}
-
-// 4D tiled tensor store shared -> global (bulk async group; out-of-range elements skipped).
-__device__ __forceinline__ void tma_store_4d(const CUtensorMap* tm, int c0, int c1, int c2, int c3,
-                                             const void* src) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3, %4}], [%5];" ::"l"(
-          reinterpret_cast<uint64_t>(tm)),
-      "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(smem_u32(src))
-      : "memory");
-}
-
-// 5D tiled tensor load / store (the y-blocked workspace: x, y in block, z, y block, component).
+// 5D tiled tensor load global -> shared (completion counted on `bar` in bytes) and store shared ->
+// global (bulk async group; out-of-range elements skipped), for the y-blocked workspace: x, y in
+// block, z, y block, component.
 __device__ __forceinline__ void tma_load_5d(void* dst, const CUtensorMap* tm, int c0, int c1, int c2, int c3, int c4,
                                             uint64_t* bar) {
   asm volatile(
@@ -163,7 +145,7 @@ __device__ __forceinline__ bool block_setup_n(const void* tile, uint64_t* bars, 
 
 // Bounded wait for phase `parity` of a tile's copies, shared by the block: every thread
 // polls; a timeout anywhere aborts the whole block (uniformly) and records an error.
-__device__ __forceinline__ bool block_wait(uint64_t* bar, int* fail, int* err, uint32_t parity, long long limit) {
+__device__ __forceinline__ bool block_wait(uint64_t* bar, int* fail, int* err, uint32_t parity, unsigned limit) {
   if (!mbar_wait(bar, parity, limit)) *fail = 1;
   __syncthreads();
   if (*fail) {

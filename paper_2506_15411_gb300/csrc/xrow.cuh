@@ -26,9 +26,9 @@
 // on shared memory, which its three or four stages cross 17 times per value, and on their bank
 // conflicts; this one crosses it 13 times with two fifths of the conflicts (275 x 275 x 315: 47 ->
 // 19 million; a quarter on rows of 640).  Update pass, staged -> rows (ms, one GB300):
-// 640 x 640 x 336 2.91 -> 2.16 (6.6 TB/s, 0.97 of a copy), 384 x 384 x 256 0.966 -> 0.62 (0.93),
-// 275 x 275 x 315 0.649 -> 0.386 (0.95), 256 x 256 x 192 0.356 -> 0.219 (0.88), 175 x 175 x 198
-// 0.163 -> 0.108 (0.86), 192 x 192 x 128 0.128 -> 0.084 (0.86), 128^3 0.076 -> 0.047; 64^3 0.0214
+// 640 x 640 x 336 2.91 -> 2.13 (6.7 TB/s, 0.99 of a copy), 384 x 384 x 256 0.966 -> 0.614 (0.94),
+// 275 x 275 x 315 0.649 -> 0.383 (0.95), 256 x 256 x 192 0.356 -> 0.220 (0.88), 175 x 175 x 198
+// 0.163 -> 0.109 (0.85), 192 x 192 x 128 0.128 -> 0.084 (0.86), 128^3 0.076 -> 0.047; 64^3 0.0214
 // -> 0.0184 (latency of one to three tiles a block).
 #pragma once
 #include <algorithm>
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
         // the set's use u is armed once the tile counts as issued: before that its mbarrier may
         // still be two phases back, where the parity alone would let the wait through
         bool on = *issued > i;
-        for (long long left = a.wait_limit; !on && !*failed && left > 0; --left) {
+        for (unsigned left = a.wait_limit; !on && !*failed && left > 0; --left) {
           __nanosleep(32);
           on = *issued > i;
         }
@@ -238,26 +238,26 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_xrow(const IterArgs a, const
           constexpr int U = 4;
           if (mode != 2) {
 #pragma unroll
-          for (int r0u = 0; r0u < R; r0u += U) {
-            float2 vv[U], ec[U];
+            for (int r0u = 0; r0u < R; r0u += U) {
+              float2 vv[U], ec[U];
 #pragma unroll
-            for (int i2 = 0; i2 < U; ++i2)
-              if (r0u + i2 < R) {
-                vv[i2] = vr[(r0u + i2) * B];
-                ec[i2] = er[(r0u + i2) * B];
-              }
+              for (int i2 = 0; i2 < U; ++i2)
+                if (r0u + i2 < R) {
+                  vv[i2] = vr[(r0u + i2) * B];
+                  ec[i2] = er[(r0u + i2) * B];
+                }
 #pragma unroll
-            for (int i2 = 0; i2 < U; ++i2)
-              if (r0u + i2 < R) {
-                const int r = r0u + i2;
-                const float2 gm = make_float2(-vv[i2].y * ie, vv[i2].x * ie);
-                const float2 d = cmul(gm, csub(ec[i2], x[r]));
-                const float2 en = csub(ec[i2], d);
-                er[r * B] = en;
-                acc = fmaf(d.x, d.x, fmaf(d.y, d.y, acc));
-                x[r] = cmul(vv[i2], en);
-              }
-          }
+              for (int i2 = 0; i2 < U; ++i2)
+                if (r0u + i2 < R) {
+                  const int r = r0u + i2;
+                  const float2 gm = make_float2(-vv[i2].y * ie, vv[i2].x * ie);
+                  const float2 d = cmul(gm, csub(ec[i2], x[r]));
+                  const float2 en = csub(ec[i2], d);
+                  er[r * B] = en;
+                  acc = fmaf(d.x, d.x, fmaf(d.y, d.y, acc));
+                  x[r] = cmul(vv[i2], en);
+                }
+            }
           }
           int y, z;
           rowdec(r0 + row, y, z);

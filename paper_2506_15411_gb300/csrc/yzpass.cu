@@ -38,9 +38,9 @@ cudaError_t yz_grid_sizes(IterArgs& a, int sms) {
   if (a.yc.sets) {   // one block per SM
     a.grid_y = std::max(1, std::min(ypass_tiles(a), sms));
   } else {
-  e = with_tx(a.tx_y, [&](auto T) { return y_occupancy<decltype(T)::value>(a, &occ); });
-  if (e != cudaSuccess) return e;
-  a.grid_y = std::max(1, std::min(ypass_tiles(a), sms * std::max(1, occ)));
+    e = with_tx(a.tx_y, [&](auto T) { return y_occupancy<decltype(T)::value>(a, &occ); });
+    if (e != cudaSuccess) return e;
+    a.grid_y = std::max(1, std::min(ypass_tiles(a), sms * std::max(1, occ)));
   }
   if (a.zc.sets) {
     a.grid_z = std::max(1, std::min(zpass_tiles(a), sms));

@@ -149,12 +149,11 @@ def columns(b, n, S, NG, copy, careless):
         k = kl = ph = 0
         ok = True
         if not copy:
-            for i in range(n):
+            for _ in range(S, n):
                 ok = yield from refill(k, ph)
                 if not ok:
                     break
-                if i + S < n:
-                    load(k)
+                load(k)
                 yield
                 k += 1
                 if k == S:
@@ -172,10 +171,13 @@ def columns(b, n, S, NG, copy, careless):
                 k += 1
                 if k == S:
                     k, ph = 0, ph ^ 1
-        if not ok:
-            yield from b.settle(full, b.issued, S)
-            while not tbar.passed(0):
-                yield
+        if not ok or b.failed:
+            yield from landed()
+
+    def landed():
+        yield from b.settle(full, b.issued, S)
+        while not tbar.passed(0):
+            yield
 
     def sync(g):
         m = meet[g]
@@ -211,6 +213,8 @@ def columns(b, n, S, NG, copy, careless):
                 yield from sync(g)
                 if w == 0:
                     done[k].arrive()
+        if not copy and b.failed:
+            yield from landed()
 
     return [loader()] + [warp(g, w) for g in range(NG) for w in range(W)], W * n
 
