@@ -253,6 +253,7 @@ int seat_begin(Batch* b, Seat& s, float2* E, const SourceArgs& src, Phase phase)
   s.run.t0 = std::chrono::steady_clock::now();
   s.run.E = E;
   s.mem.src = src;
+  s.mem.phase = 0;
   s.blk = 0;
   const size_t Nw = p->base.Nw;
   CK(cudaMemsetAsync(p->Ei + (size_t)s.idx * 3 * Nw, 0, 3 * Nw * sizeof(float2), b->stream));

@@ -97,3 +97,27 @@ def test_blocks_longer_than_the_ring_of_residuals():
     r = ref.history[-1] / ref.history[0]
     assert abs(out[0][1] - r) <= 1e-4 * r
     assert np.linalg.norm(out[0][0].cpu().numpy() - ref.E) <= 2e-5 * np.linalg.norm(ref.E)
+
+
+def test_a_served_adjoint_starts_its_twiddle_tables_anew():
+    """Blocks of 12 iterations: the forward series ends at the fifth of eight tables, and the adjoint begins
+    at the first, as it does through a plan."""
+    import torch
+
+    from paper_2506_15411_gb300 import CBSPlan, PlaneWave
+    from paper_2506_15411_gb300.serve import GridSpec, Server
+    nx, ny, nz = 40, 36, 44
+    pads = (5, 5, 5)
+    r0 = (nx // 2, ny // 2, nz // 2)
+    dev = torch.from_numpy(inputs.random_eps(nx, ny, nz, seed=10)).cuda()
+    with CBSPlan(nx, ny, nz, LAM / 8, LAM, 1.0, pads, pads, tol=0.0, max_iter=20, check_every=12) as plan:
+        plan.set_permittivity(dev)
+        E, _ = plan.forward(PlaneWave())
+        Ea, _ = plan.adjoint(r0, E)
+        grad, _ = plan.gradient(E, Ea, r0)
+    with Server(max_active=2, tol=0.0, max_iter=20, check_every=12) as srv:
+        spec = GridSpec(nx, ny, nz, LAM / 8, LAM, 1.0, pads, pads)
+        for t in range(2):
+            srv.submit(spec, dev, PlaneWave(), r0, adjoint=True, want_field=True, want_grad=True, tag=t)
+        for r in srv.wait(2):
+            assert torch.equal(r.E, E) and torch.equal(r.grad, grad)
